@@ -25,7 +25,7 @@ void count_launch(int64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed
 
 void Scratch::release_all()
 {
-    DevBuf *all[] = {&keys, &vals, &skeys, &svals, &cub, &desc, &tmaps, &active, &flags, &surv, &ekeys, &surv_sorted,
+    DevBuf *all[] = {&keys, &ranks, &order, &bin_table, &cub, &desc, &tmaps, &active, &flags, &surv, &ekeys, &surv_sorted,
                      &pos, &cellk, &celli, &cellk_s, &celli_s, &cell_start, &stat, &acc, &cells, &counters};
     for (DevBuf *b : all) b->release();
     lsets.release();
@@ -289,8 +289,9 @@ extern "C" void ac_destroy_volume(ac_volume *vol) { ac::destroy_volume_on(vol, n
 
 // ------------------------------------------------------------------ seeding
 __global__ void seed_lattice_kernel(float *state, int64_t C, int Lx, int Ly, float fx, float fy, float fz,
-                                    float stride, float R0, int ndim)
+                                    float stride, float R0, int ndim, int32_t *hold, int32_t *status)
 {
+    if (blockIdx.x == 0 && threadIdx.x < 4) status[threadIdx.x] = 0;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < C; k += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = k % Lx, j = (k / Lx) % Ly, l = k / ((int64_t)Lx * Ly);
         state[k] = fmaf((float)i, stride, fx);
@@ -298,6 +299,7 @@ __global__ void seed_lattice_kernel(float *state, int64_t C, int Lx, int Ly, flo
         state[2 * C + k] = ndim == 3 ? fmaf((float)l, stride, fz) : 0.0f;
         state[3 * C + k] = R0;
         state[4 * C + k] = 0.0f;
+        hold[k] = 0;
     }
 }
 
@@ -438,11 +440,9 @@ extern "C" ac_status ac_reseed(ac_contours *c, void *cuda_stream)
     const int threads = 256;
     const int64_t C = c->C;
     const int64_t blocks = std::min<int64_t>((C + threads - 1) / threads, 1 << 16);
-    AC_CUDA(cudaMemsetAsync(c->status, 0, sizeof(int32_t) * 4, st));
-    AC_CUDA(cudaMemsetAsync(c->hold, 0, sizeof(int32_t) * (size_t)(C > 0 ? C : 1), st));
     seed_lattice_kernel<<<(unsigned)blocks, threads, 0, st>>>(c->state, C, (int)c->L[0], (int)c->L[1], c->first[0],
                                                               c->first[1], c->first[2], c->stride, c->R0,
-                                                              c->vol->ndim);
+                                                              c->vol->ndim, c->hold, c->status);
     count_launch();
     AC_CUDA(cudaGetLastError());
     return AC_OK;
@@ -758,28 +758,6 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
     AC_FAIL(AC_ERR_ARG, "ac_evolve: staged region cannot fit the shared-memory budget; use smaller bricks");
 }
 
-__global__ void bin_kernel(const VolDesc *vols, int n_vols, int64_t total, int3 B, uint32_t *keys, uint32_t *vals)
-{
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x) {
-        int v = 0;
-        for (int i = 1; i < n_vols; ++i)
-            if (vols[i].contour_base <= g) v = i;
-        const VolDesc &V = vols[v];
-        const int64_t k = g - V.contour_base;
-        const int Bd[3] = {B.x, B.y, B.z};
-        int bi[3];
-        for (int d = 0; d < 3; ++d) {
-            const float c = V.state[d * V.C + k];
-            int idx = (int)floorf(c * V.inv_sp[d]);
-            idx = idx < 0 ? 0 : (idx >= V.n[d] ? V.n[d] - 1 : idx);
-            int b = idx / Bd[d];
-            bi[d] = b >= V.nb[d] ? V.nb[d] - 1 : b;
-        }
-        keys[g] = (uint32_t)(V.brick_base + bi[0] + (int64_t)V.nb[0] * (bi[1] + (int64_t)V.nb[1] * bi[2]));
-        vals[g] = (uint32_t)g;
-    }
-}
-
 CUtensorMapDataType tma_type(ac_dtype t)
 {
     switch (t) {
@@ -830,8 +808,7 @@ struct Prepared {
     ac_dtype dtype = AC_U8;
     int n_sets = 0;
     int64_t total = 0, bricks = 0;
-    int end_bit = 1;
-    size_t cub_bytes = 0;
+    BinSpace bin{};
     std::vector<VolDesc> desc;
     std::vector<CUtensorMap> maps;
     ac_contours *owner = nullptr;   // status word, path counters, kernel-time events
@@ -1058,20 +1035,20 @@ ac_status prepare_sets(ac_contours *const *sets, const ac_batch_item *items, int
     CUtensorMap *dmaps = reinterpret_cast<CUtensorMap *>(((uintptr_t)sc.tmaps.p + 127) & ~(uintptr_t)127);
     AC_CUDA(cudaMemcpyAsync(dmaps, pr.maps.data(), sizeof(CUtensorMap) * n_sets, cudaMemcpyHostToDevice, st));
 
-    // binning and sort space
+    // binning space
+    pr.bin.sort = bin_by_sort(total, bricks);
+    AC_CUDA(bin_table_bytes(total, bricks, pr.bin.sort, &pr.bin.table_bytes));
     AC_CUDA(sc.keys.ensure(sizeof(uint32_t) * total));
-    AC_CUDA(sc.vals.ensure(sizeof(uint32_t) * total));
-    AC_CUDA(sc.skeys.ensure(sizeof(uint32_t) * total));
-    AC_CUDA(sc.svals.ensure(sizeof(uint32_t) * total));
-    pr.end_bit = 1;
-    while (((int64_t)1 << pr.end_bit) < bricks + 1) ++pr.end_bit;
-    AC_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, pr.cub_bytes, sc.keys.as<uint32_t>(), sc.skeys.as<uint32_t>(),
-                                            sc.vals.as<uint32_t>(), sc.svals.as<uint32_t>(), (int)total, 0, pr.end_bit, st));
-    AC_CUDA(sc.cub.ensure(pr.cub_bytes));
+    AC_CUDA(sc.ranks.ensure(sizeof(uint32_t) * total));
+    AC_CUDA(sc.order.ensure(sizeof(uint32_t) * total));
+    AC_CUDA(sc.bin_table.ensure(pr.bin.table_bytes));
+    pr.bin.table = sc.bin_table.p;
+    pr.bin.keys = sc.keys.as<uint32_t>();
+    pr.bin.ranks = sc.ranks.as<uint32_t>();
+    pr.bin.order = sc.order.as<uint32_t>();
 
     a.tmaps = dmaps;
-    a.sorted_brick = sc.skeys.as<uint32_t>();
-    a.sorted_gidx = sc.svals.as<uint32_t>();
+    bin_bind(a, pr.bin);
     a.total_bricks = bricks;
     for (int d = 0; d < 3; ++d) {
         a.B[d] = pl.B[d];
@@ -1091,10 +1068,7 @@ __global__ void compact_active_kernel(const VolDesc *vols, int n_vols, int64_t t
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gi < total; gi += stride) {
-        int v = 0;
-        for (int i = 1; i < n_vols; ++i)
-            if (vols[i].contour_base <= gi) v = i;
-        const VolDesc &V = vols[v];
+        const VolDesc &V = vols[find_set(vols, n_vols, gi)];
         const int64_t k = gi - V.contour_base;
         const bool run = V.first_iter <= V.last_iter && !(V.hold && (V.hold[k] & HOLD_STOPPED));
         // one atomic per warp: the lanes of this iteration share a block of the list
@@ -1120,7 +1094,7 @@ ac_status enqueue_prepared(Prepared &pr, Scratch &sc, cudaStream_t st, int64_t *
     EvolveArgs a = pr.a;
     ac_contours *owner = pr.owner;
     int64_t nl = 0;
-    AC_CUDA(cudaMemsetAsync(owner->path_counts, 0, sizeof(unsigned long long) * 3, st));
+    if (!pr.pl.brick) AC_CUDA(cudaMemsetAsync(owner->path_counts, 0, sizeof(unsigned long long) * 3, st));
     if (pr.pl.grid) {
         const int64_t per_cta = (int64_t)pr.pl.warps * 32 / pr.pl.G;
         const int64_t grid = std::min<int64_t>((pr.total + per_cta - 1) / per_cta, (int64_t)1 << 30);
@@ -1141,16 +1115,7 @@ ac_status enqueue_prepared(Prepared &pr, Scratch &sc, cudaStream_t st, int64_t *
         }
         AC_CUDA(cudaEventRecordWithFlags(owner->ev1, st, ev_flags));
     } else {
-        const int64_t blocks = std::min<int64_t>((pr.total + 255) / 256, 1 << 16);
-        bin_kernel<<<(unsigned)blocks, 256, 0, st>>>(a.vols, pr.n_sets, pr.total,
-                                                     make_int3(pr.pl.B[0], pr.pl.B[1], pr.pl.B[2]),
-                                                     sc.keys.as<uint32_t>(), sc.vals.as<uint32_t>());
-        ++nl;
-        AC_CUDA(cudaGetLastError());
-        size_t tmp = pr.cub_bytes;
-        AC_CUDA(cub::DeviceRadixSort::SortPairs(sc.cub.p, tmp, sc.keys.as<uint32_t>(), sc.skeys.as<uint32_t>(),
-                                                sc.vals.as<uint32_t>(), sc.svals.as<uint32_t>(), (int)pr.total, 0,
-                                                pr.end_bit, st));
+        AC_CUDA(launch_bin(a, pr.bin, st, &nl));
         AC_CUDA(cudaEventRecordWithFlags(owner->ev0, st, ev_flags));
         cudaError_t e = launch_evolve(pr.dtype, a, pr.pl, pr.bricks, st);
         if (e != cudaSuccess) AC_FAIL(AC_ERR_CUDA, std::string("ac_evolve: brick launch: ") + cudaGetErrorString(e));
@@ -1209,9 +1174,9 @@ ac_status ac::check_evolve_params(const ac_evolve_params *p) { return check_para
 // ------------------------------------------------------------------ allocation-free evolve
 // One file-scope device array holds every temporary of ac_evolve_static.  Byte
 // layout: [0, 16) status word, [64, 96) path counters, [256, ...) volume
-// descriptor, [512, 640) TMA descriptor, [1024, ...) binning keys, contour indices
-// and their sorted copies (4 x 4 bytes per contour), then the sort's temporary
-// space up to the end of the array.
+// descriptor, [512, 640) TMA descriptor, [1024, ...) binning keys, ranks and contour
+// indices (3 x 4 bytes per contour), then the table of brick ranges (or the sorted
+// keys and the sort's temporary space) up to the end of the array.
 static __device__ __align__(256) unsigned char g_static_scratch[AC_STATIC_SCRATCH_BYTES];
 
 namespace {
@@ -1440,34 +1405,33 @@ extern "C" ac_status ac_evolve_static(const void *volume_dev, ac_dtype dtype, in
             AC_FAIL(AC_ERR_CUDA, "ac_evolve_static: cuTensorMapEncodeTiled failed (code " + std::to_string((int)r) + ")");
         CUtensorMap *dmap = reinterpret_cast<CUtensorMap *>(base + kStaticTmap);
         AC_CUDA(cudaMemcpyAsync(dmap, &map, sizeof(map), cudaMemcpyHostToDevice, st));
-        uint32_t *keys = reinterpret_cast<uint32_t *>(base + kStaticArrays);
-        uint32_t *vals = keys + AC_STATIC_MAX_CONTOURS;
-        uint32_t *skeys = vals + AC_STATIC_MAX_CONTOURS;
-        uint32_t *svals = skeys + AC_STATIC_MAX_CONTOURS;
-        unsigned char *tmp_space = reinterpret_cast<unsigned char *>(svals + AC_STATIC_MAX_CONTOURS);
-        const size_t tmp_cap = (size_t)AC_STATIC_SCRATCH_BYTES - (size_t)(tmp_space - base);
-        int end_bit = 1;
-        while (((int64_t)1 << end_bit) < bricks + 1) ++end_bit;
-        size_t tmp = 0;
-        AC_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tmp, keys, skeys, vals, svals, (int)n_contours, 0, end_bit, st));
-        if (tmp > tmp_cap)
-            AC_FAIL(AC_ERR_BUDGET, "ac_evolve_static: the sort needs " + std::to_string(tmp) +
+        // keys, ranks and order, then the table, in the rest of the array
+        BinSpace bin{};
+        bin.keys = reinterpret_cast<uint32_t *>(base + kStaticArrays);
+        bin.ranks = bin.keys + AC_STATIC_MAX_CONTOURS;
+        bin.order = bin.ranks + AC_STATIC_MAX_CONTOURS;
+        bin.table = bin.order + AC_STATIC_MAX_CONTOURS;
+        const size_t cap = (size_t)AC_STATIC_SCRATCH_BYTES - (size_t)((unsigned char *)bin.table - base);
+        bin.sort = bin_by_sort(n_contours, bricks);
+        AC_CUDA(bin_table_bytes(n_contours, bricks, bin.sort, &bin.table_bytes));
+        if (!bin.sort && bin.table_bytes > cap) {   // a sorted list needs no space per brick
+            bin.sort = true;
+            AC_CUDA(bin_table_bytes(n_contours, bricks, bin.sort, &bin.table_bytes));
+        }
+        if (bin.table_bytes > cap)
+            AC_FAIL(AC_ERR_BUDGET, "ac_evolve_static: the sort needs " + std::to_string(bin.table_bytes) +
                                        " bytes of temporary space, more than the static array holds");
-        const int64_t blocks = std::min<int64_t>((n_contours + 255) / 256, 1 << 16);
-        bin_kernel<<<(unsigned)blocks, 256, 0, st>>>(ddesc, 1, n_contours, make_int3(pl.B[0], pl.B[1], pl.B[2]), keys,
-                                                     vals);
-        count_launch();
-        AC_CUDA(cudaGetLastError());
-        AC_CUDA(cub::DeviceRadixSort::SortPairs(tmp_space, tmp, keys, skeys, vals, svals, (int)n_contours, 0, end_bit, st));
         a.tmaps = dmap;
-        a.sorted_brick = skeys;
-        a.sorted_gidx = svals;
+        bin_bind(a, bin);
         a.total_bricks = bricks;
         for (int d = 0; d < 3; ++d) {
             a.B[d] = pl.B[d];
             a.halo[d] = pl.halo[d];
             a.ext[d] = pl.ext[d];
         }
+        int64_t nl = 0;
+        AC_CUDA(launch_bin(a, bin, st, &nl));
+        count_launch(nl);
         a.raw_bytes = pl.raw;
         a.quad_off = pl.quad_off;
         a.smem_bytes = pl.smem;

@@ -710,14 +710,6 @@ __device__ __forceinline__ Step eval_contour(const Gather &gat, const IterC<DIM>
     return finish<DIM>(sums, R, a, scale);
 }
 
-__device__ __forceinline__ int find_vol(const EvolveArgs &a, int64_t idx, bool by_brick)
-{
-    int v = 0;
-    for (int i = 1; i < a.n_vols; ++i)
-        if ((by_brick ? a.vols[i].brick_base : a.vols[i].contour_base) <= idx) v = i;
-    return v;
-}
-
 __device__ __forceinline__ int64_t lower_bound_u32(const uint32_t *keys, int64_t n, uint32_t key)
 {
     int64_t lo = 0, hi = n;
@@ -729,6 +721,8 @@ __device__ __forceinline__ int64_t lower_bound_u32(const uint32_t *keys, int64_t
 }
 
 // ----------------------------------------------------------------- brick kernel
+constexpr int LIST_MAX = 128;   // contours of a brick that are ordered by index in shared memory
+
 // One CTA per brick: TMA stages the brick plus halo into shared memory once (2D:
 // then rewritten as quads so one shared-memory load feeds a bilinear sample);
 // each group of G lanes evolves one contour of the brick through all iterations
@@ -746,11 +740,18 @@ __global__ void __maxnreg__(DIM == 2 ? 96 : 128) evolve_brick_kernel(const __gri
     using QT = typename QuadOf<T>::type;
 
     const int64_t b = blockIdx.x;
-    const int64_t cb = lower_bound_u32(a.sorted_brick, a.total_contours, (uint32_t)b);
-    const int64_t ce = lower_bound_u32(a.sorted_brick, a.total_contours, (uint32_t)(b + 1));
+    int64_t cb, ce;
+    if (a.ranges) {
+        const uint2 r = a.ranges[b];
+        cb = r.x;
+        ce = cb + r.y;
+    } else {
+        cb = lower_bound_u32(a.sorted_brick, a.total_contours, (uint32_t)b);
+        ce = lower_bound_u32(a.sorted_brick, a.total_contours, (uint32_t)(b + 1));
+    }
     if (cb == ce) return;   // empty brick (uniform over the CTA)
 
-    const int v = find_vol(a, b, true);
+    const int v = find_set<&VolDesc::brick_base>(a.vols, a.n_vols, b);
     const VolDesc &V = a.vols[v];
     if (V.first_iter > V.last_iter) return;   // no iterations for this set in this launch
     const int64_t lb = b - V.brick_base;
@@ -765,13 +766,29 @@ __global__ void __maxnreg__(DIM == 2 ? 96 : 128) evolve_brick_kernel(const __gri
     // One thread issues the load and decides whether it landed within the bound, so
     // every thread of the CTA takes the same branch.  On giving up it records the
     // timeout and waits (again bounded) for the copy in flight, so that no copy is
-    // still writing shared memory when the CTA exits.
+    // still writing shared memory when the CTA exits.  While the copy runs, the brick's
+    // contours are put in increasing order (each counts the smaller ones): neighbours
+    // share a warp, and with it a gather path, and the path counts do not depend on the
+    // order in which the contours were grouped.  A longer list stays as it is.
     __shared__ int landed;
-    if (threadIdx.x == 0) mbar_init(&mbar, 1);
-    __syncthreads();
+    __shared__ uint32_t list[LIST_MAX];
     if (threadIdx.x == 0) {
+        mbar_init(&mbar, 1);
         mbar_expect_tx(&mbar, (uint32_t)a.raw_bytes);
         tma_load_3d(smem_raw, &a.tmaps[v], r0[0], r0[1], r0[2], &mbar);
+    }
+    if (ce - cb <= LIST_MAX) {
+        const int n = (int)(ce - cb);
+        for (int i = threadIdx.x; i < n; i += blockDim.x) list[i] = a.order[cb + i];
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            const uint32_t g = list[i];
+            int rank = 0;
+            for (int j = 0; j < n; ++j) rank += list[j] < g ? 1 : 0;
+            a.order[cb + rank] = g;
+        }
+    }
+    if (threadIdx.x == 0) {
         landed = mbar_wait_bounded(&mbar, 0, a.tma_polls) ? 1 : 0;
         if (!landed) {
             atomicOr(V.status, STATUS_TMA_TIMEOUT);
@@ -827,7 +844,7 @@ __global__ void __maxnreg__(DIM == 2 ? 96 : 128) evolve_brick_kernel(const __gri
         int64_t k = 0;
         int32_t h = 0;
         if (live) {
-            k = (int64_t)a.sorted_gidx[i] - V.contour_base;
+            k = (int64_t)a.order[i] - V.contour_base;
             h = V.hold ? V.hold[k] : 0;
             live = !(h & HOLD_STOPPED);   // stopped by a rule in an earlier call
         }
@@ -968,7 +985,7 @@ __global__ void __launch_bounds__(256) evolve_plain_kernel(const __grid_constant
     const int64_t items = a.active ? (int64_t)*a.n_active : a.total_contours;
     for (int64_t it = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G; it < items; it += groups) {
         const int64_t gi = a.active ? (int64_t)a.active[it] : it;
-        const int v = find_vol(a, gi, false);
+        const int v = find_set(a.vols, a.n_vols, gi);
         const VolDesc &V = a.vols[v];
         if (n < V.first_iter || n > V.last_iter) continue;   // outside this set's iterations
         const int64_t k = gi - V.contour_base;

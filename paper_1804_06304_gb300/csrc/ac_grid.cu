@@ -117,7 +117,7 @@ __global__ void __maxnreg__(80) evolve_grid_kernel(const __grid_constant__ Evolv
     const unsigned mask = group_mask<G>();
     const int64_t groups = (int64_t)gridDim.x * (blockDim.x / G);
     for (int64_t gi = (int64_t)blockIdx.x * (blockDim.x / G) + threadIdx.x / G; gi < a.total_contours; gi += groups) {
-        const int v = find_vol(a, gi, false);
+        const int v = find_set(a.vols, a.n_vols, gi);
         const VolDesc &V = a.vols[v];
         if (V.first_iter > V.last_iter) continue;   // no iterations for this set in this launch
         const int64_t k = gi - V.contour_base;

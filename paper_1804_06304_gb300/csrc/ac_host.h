@@ -6,6 +6,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <string>
 
 #include "ac_internal.cuh"
@@ -79,9 +80,9 @@ struct HostBuf {
 };
 
 struct Scratch {
-    DevBuf keys, vals, skeys, svals, cub, desc, tmaps, active;       // evolve
+    DevBuf keys, ranks, order, bin_table, desc, tmaps, active;       // evolve
     DevBuf flags, surv, ekeys, surv_sorted, pos, cellk, celli, cellk_s, celli_s, cell_start, stat, acc,
-        cells, counters;                                               // localize
+        cells, counters, cub;                                          // localize
     DevBuf lsets, und;                                                 // localize: set descriptors, open counts
     HostBuf hcount, hcells, hsets;                                     // localize: read back / uploaded
     void release_all();
@@ -135,6 +136,20 @@ cudaError_t launch_evolve_f32(const EvolveArgs &a, bool brick, int G, bool comp,
 
 // the voxel-grid form of Eq. 5 (ac_grid.cu)
 cudaError_t launch_grid(ac_dtype t, const EvolveArgs &a, int G, bool comp, int warps, int64_t grid, cudaStream_t st);
+
+// Space for grouping a launch's contours by brick (ac_bin.cu): keys, ranks and order
+// hold one word per contour, `table` (16-byte aligned) what bin_table_bytes says for
+// the chosen form (`sort`: sorted list, else ranges per brick).
+struct BinSpace {
+    bool sort;
+    void *table;
+    size_t table_bytes;
+    uint32_t *keys, *ranks, *order;
+};
+bool bin_by_sort(int64_t total, int64_t bricks);
+cudaError_t bin_table_bytes(int64_t total, int64_t bricks, bool sort, size_t *bytes);
+void bin_bind(EvolveArgs &a, const BinSpace &s);   // the brick kernel's view of the result
+cudaError_t launch_bin(const EvolveArgs &a, const BinSpace &s, cudaStream_t st, int64_t *launches);
 
 // the argument checks of ac_evolve (ac_api.cu)
 ac_status check_evolve_params(const ac_evolve_params *p);
