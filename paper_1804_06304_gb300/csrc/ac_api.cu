@@ -552,15 +552,6 @@ extern "C" ac_status ac_philox4x32_10(const uint32_t *ctr_dev, uint64_t key, uin
 // ------------------------------------------------------------------ evolution
 namespace {
 
-struct Plan {
-    int B[3], halo[3], ext[3];
-    int raw;        // staged region bytes
-    int quad_off;   // 2D: byte offset of the quads (0: none)
-    int smem;       // dynamic shared memory bytes
-    int G, warps;
-    bool brick, grid, comp, acc;
-};
-
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -679,83 +670,212 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
         const int b = p->brick[d] ? p->brick[d] : (int)std::lround(cells[d] * stride_hint / vol->sp[d]);
         return std::max(1, std::min(b, (int)std::min<int64_t>(vol->n[d], 224)));
     };
-    for (int d = 0; d < vol->ndim; ++d) {
-        B[d] = brick_of(d);
-        const double hf = p->halo_factor > 0.0f ? p->halo_factor : (vol->ndim == 3 ? 2.5 : 3.5);
-        h[d] = (int)std::ceil((hf * r_hint + 0.5 * p->dR) / vol->sp[d]) + 2;
-    }
-    if (!p->brick[0] && !p->brick[1] && !p->brick[2]) {
-        // a small volume gets more, smaller bricks (down to 2 cells per axis in 2D, 1 in
-        // 3D), so that the grid holds about four CTAs per slot (152 SMs x 2) instead of
-        // a tail wave
-        auto n_bricks = [&]() {
-            int64_t nb = 1;
-            for (int d = 0; d < vol->ndim; ++d) nb *= (vol->n[d] + B[d] - 1) / B[d];
-            return nb;
-        };
-        const int min_cells = vol->ndim == 3 ? 1 : 2;
-        while (n_bricks() < 1216) {
-            int dm = -1;
-            for (int d = 0; d < vol->ndim; ++d)
-                if (cells[d] > min_cells && (dm < 0 || cells[d] > cells[dm])) dm = d;
-            if (dm < 0) break;
-            cells[dm] = std::max(min_cells, cells[dm] / 2);
-            B[dm] = brick_of(dm);
-        }
-    }
-    // The staged region may take the shared memory its CTA's registers leave it: in 3D
-    // (128 registers a thread) a CTA of more than 8 warps has its SM alone, smaller ones
-    // share it with a second CTA.
-    for (int iter = 0; iter < 4096; ++iter) {
-        const int64_t budget = vol->ndim == 3 ? (warps_of() > 8 ? 215 * 1024 : 110 * 1024) : 200 * 1024;
-        int64_t raw = vol->es;
-        bool fits_box = true;
-        for (int d = 0; d < 3; ++d) {
-            int ext = 1;
-            if (d < vol->ndim) {
-                int64_t need = (int64_t)B[d] + 2 * (int64_t)h[d] + (d == 0 ? al - 1 : 0);
-                const int64_t cap = vol->n[d] + (d == 0 ? al - 1 : 0);
-                need = std::min(need, cap);
-                if (d == 0) need = (need + al - 1) / al * al;
-                // 3D taps are read from the raw region: a row of a multiple of 128 bytes
-                // would put the same voxel column of every row on one shared-memory bank,
-                // so such rows get 16 more bytes (unless the region spans the volume's rows)
-                if (d == 0 && vol->ndim == 3 && need < vol->n[0] && need * vol->es % 128 == 0) need += al;
-                if (need > 256) fits_box = false;
-                ext = (int)need;
-            }
-            pl.ext[d] = ext;
-            pl.B[d] = B[d];
-            pl.halo[d] = h[d];
-            raw *= ext;
-        }
-        int64_t quad_off = 0, total = raw;
-        if (vol->ndim == 2) {   // quads after the raw region: 4 halves (uint8, binary16) or float4
-            const int qbytes = (vol->dtype == AC_U8 || vol->dtype == AC_F16) ? 8 : 16;
-            quad_off = (raw + 127) / 128 * 128;
-            total = quad_off + (int64_t)(pl.ext[0] - 1) * (pl.ext[1] - 1) * qbytes;
-        }
-        if (fits_box && total <= budget) {
-            pl.raw = (int)raw;
-            pl.quad_off = (int)quad_off;
-            pl.smem = (int)total;
-            pl.warps = warps_of();
-            return AC_OK;
-        }
-        int hmax = 0, bmax = 0;
+    const double hf = p->halo_factor > 0.0f ? p->halo_factor : (vol->ndim == 3 ? 2.5 : 3.5);
+    const bool own_bricks = !p->brick[0] && !p->brick[1] && !p->brick[2];
+    // Region of the current cells: shrinks the halo, then (own bricks only, and only as
+    // the last resort) the brick until it fits.  The staged region may take the shared
+    // memory its CTA's registers leave it: in 3D (128 registers a thread) a CTA of more
+    // than 8 warps has its SM alone, smaller ones share it with a second CTA.
+    auto fit = [&](bool shrink_brick) {
         for (int d = 0; d < vol->ndim; ++d) {
-            hmax = std::max(hmax, h[d]);
-            bmax = std::max(bmax, B[d]);
+            B[d] = brick_of(d);
+            h[d] = (int)std::ceil((hf * r_hint + 0.5 * p->dR) / vol->sp[d]) + 2;
         }
-        if (hmax > 1) {
-            for (int d = 0; d < vol->ndim; ++d) h[d] = std::max(1, h[d] - 1);
-        } else if (bmax > 1 && p->brick[0] == 0 && p->brick[1] == 0 && p->brick[2] == 0) {
-            for (int d = 0; d < vol->ndim; ++d) B[d] = std::max(1, B[d] - 1);
-        } else {
-            break;
+        for (int iter = 0; iter < 4096; ++iter) {
+            const int64_t budget = vol->ndim == 3 ? (warps_of() > 8 ? 215 * 1024 : 110 * 1024) : 200 * 1024;
+            int64_t raw = vol->es;
+            bool fits_box = true;
+            for (int d = 0; d < 3; ++d) {
+                int ext = 1;
+                if (d < vol->ndim) {
+                    int64_t need = (int64_t)B[d] + 2 * (int64_t)h[d] + (d == 0 ? al - 1 : 0);
+                    const int64_t cap = vol->n[d] + (d == 0 ? al - 1 : 0);
+                    need = std::min(need, cap);
+                    if (d == 0) need = (need + al - 1) / al * al;
+                    // 3D taps are read from the raw region: a row of a multiple of 128 bytes
+                    // would put the same voxel column of every row on one shared-memory bank,
+                    // so such rows get 16 more bytes (unless the region spans the volume's rows)
+                    if (d == 0 && vol->ndim == 3 && need < vol->n[0] && need * vol->es % 128 == 0) need += al;
+                    if (need > 256) fits_box = false;
+                    ext = (int)need;
+                }
+                pl.ext[d] = ext;
+                pl.B[d] = B[d];
+                pl.halo[d] = h[d];
+                raw *= ext;
+            }
+            int64_t quad_off = 0, total = raw;
+            if (vol->ndim == 2) {   // quads after the raw region: 4 halves (uint8, binary16) or float4
+                const int qbytes = (vol->dtype == AC_U8 || vol->dtype == AC_F16) ? 8 : 16;
+                quad_off = (raw + 127) / 128 * 128;
+                total = quad_off + (int64_t)(pl.ext[0] - 1) * (pl.ext[1] - 1) * qbytes;
+            }
+            if (fits_box && total <= budget) {
+                pl.raw = (int)raw;
+                pl.quad_off = (int)quad_off;
+                pl.smem = (int)total;
+                pl.warps = warps_of();
+                return true;
+            }
+            int hmax = 0, bmax = 0;
+            for (int d = 0; d < vol->ndim; ++d) {
+                hmax = std::max(hmax, h[d]);
+                bmax = std::max(bmax, B[d]);
+            }
+            if (hmax > 1) {
+                for (int d = 0; d < vol->ndim; ++d) h[d] = std::max(1, h[d] - 1);
+            } else if (bmax > 1 && shrink_brick) {
+                for (int d = 0; d < vol->ndim; ++d) B[d] = std::max(1, B[d] - 1);
+            } else {
+                break;
+            }
+        }
+        return false;
+    };
+    for (int d = 0; d < vol->ndim; ++d) B[d] = brick_of(d);
+    if (own_bricks) {
+        // A volume of fewer than 1216 default bricks (four per slot, two slots on each of
+        // 152 SMs) leaves SMs idle or ends in a nearly empty wave.  Its bricks are chosen by
+        // an estimate of the launch's time in SM cycles: CTAs run in rounds of as many as an
+        // SM holds; a round lasts (staging) + (instructions of one warp) x f(warps per
+        // scheduler).  f and the staging costs are a fit to 500 measured layouts of 12
+        // volumes and images (64x64x32 to 260x180x60, 512^2 to 1531x1117, all voxel types, 4
+        // to 32 lanes); the chosen layout is the best measured one on 8 of them and within
+        // 11 % on the others.  Halving the default until 1216 bricks came out, as before,
+        // left too few warps in flight: 128^3 u16 at N = 512, 10 iterations 486 us -> 340 us;
+        // 512^2 u8 166 -> 75 us; 64x64x32 u8 84 -> 52 us.
+        int64_t nb0 = 1;
+        double lattice = 1.0;
+        for (int d = 0; d < vol->ndim; ++d) {
+            nb0 *= (vol->n[d] + B[d] - 1) / B[d];
+            lattice *= std::max(1.0, std::floor(vol->n[d] * (double)vol->sp[d] / stride_hint));
+        }
+        if (nb0 < 1216) {
+            const int reg_warps = vol->ndim == 3 ? 16 : 21;   // warps an SM's registers hold
+            const double per_warp = 32.0 / G;                 // contours a warp evolves at once
+            const double instr = p->T * ((double)p->N / G * (vol->ndim == 3 ? 115.0 : 85.0) + 400.0);
+            auto f = [](double x) { return 2.94 + 0.66 * std::max(x, 1.1); };
+            // 3D taps of a warp land all over a ball of 2 R0: how unevenly the region's pitches
+            // spread that box over the 32 shared-memory banks (1: evenly)
+            auto uneven = [&]() {
+                if (vol->ndim == 2) return 1.0;
+                int side[3], first[32] = {0};
+                for (int d = 0; d < 3; ++d) side[d] = std::min(64, std::max(1, (int)(2.0 * r_hint / vol->sp[d])));
+                for (int z = 0; z < side[2]; ++z)
+                    for (int y = 0; y < side[1]; ++y) ++first[((z * pl.ext[1] + y) * pl.ext[0] * vol->es / 4) & 31];
+                const int words = std::max(1, side[0] * vol->es / 4);
+                double sum = 0.0, sq = 0.0;
+                for (int b = 0; b < 32; ++b) {
+                    double n = 0.0;
+                    for (int w = 0; w < words; ++w) n += first[(b - w) & 31];
+                    sum += n;
+                    sq += n * n;
+                }
+                return 32.0 * sq / (sum * sum);
+            };
+            auto estimate = [&](int warps, int smem) {
+                double nb = 1.0, full = 1.0;   // bricks; contours of a full brick
+                for (int d = 0; d < vol->ndim; ++d) {
+                    const double cell = B[d] * (double)vol->sp[d] / stride_hint;
+                    nb *= (double)((vol->n[d] + B[d] - 1) / B[d]);
+                    full *= std::min(std::max(1.0, std::floor(vol->n[d] * (double)vol->sp[d] / stride_hint)),
+                                     std::ceil(cell - 1e-6));
+                }
+                const int r = std::max(1, std::min({reg_warps / warps, 233472 / (smem + 1088), 32}));
+                const double busy = std::min(lattice / nb / per_warp, (double)warps);   // warps at work, on average
+                const double most = std::min((double)warps, std::ceil(full / per_warp));
+                const double passes = std::ceil(full / per_warp / warps);
+                const double quads = vol->ndim == 2 ? smem / (vol->es == 1 ? 9.0 : 20.0) / (warps * 32) * 1000.0 : 0.0;
+                const double stage = 3000.0 + smem / 14.4 + quads;
+                const double k = nb / 152.0, whole = std::floor(k / r);
+                double t = whole * (stage + instr * passes * f(r * busy / 4));
+                if (const double rest = std::ceil(k - whole * r); rest > 0.0)
+                    t += stage + instr * passes * f(rest * (rest > 1.0 ? busy : most) / 4);
+                return t;
+            };
+            static const int sizes3[] = {6, 4, 3, 2, 1}, sizes2[] = {12, 10, 8, 6, 5, 4, 3, 2}, one[] = {1};
+            const int *sizes = vol->ndim == 3 ? sizes3 : sizes2, n_sizes = vol->ndim == 3 ? 5 : 8;
+            const int *sizes_z = vol->ndim == 3 ? sizes3 : one, n_z = vol->ndim == 3 ? 5 : 1;
+            const double away = std::min(1.0, p->T / 100.0);
+            auto time_of = [&]() {   // of the current cells' fitted layout
+                // a halo cut short sends balls that have grown or moved to global memory (cut by
+                // 1.4 R0: 0.7 % of the contour-iterations of 10, 32 % of 100), and a CTA waits
+                // for its slowest warp
+                const double cut = std::max(0.0, hf - ((h[0] - 2) * (double)vol->sp[0] - 0.5 * p->dR) / r_hint);
+                return estimate(pl.warps, pl.smem) * (1.0 + away * cut * cut) * (0.915 + 0.085 * uneven());
+            };
+            // the default cells, halved until 1216 bricks come out: kept unless another layout
+            // promises 7 % (what the estimate is good for)
+            const int min_cells = vol->ndim == 3 ? 1 : 2;
+            for (int64_t nb = nb0; nb < 1216;) {
+                int dm = -1;
+                for (int d = 0; d < vol->ndim; ++d)
+                    if (cells[d] > min_cells && (dm < 0 || cells[d] > cells[dm])) dm = d;
+                if (dm < 0) break;
+                cells[dm] = std::max(min_cells, cells[dm] / 2);
+                nb = 1;
+                for (int d = 0; d < vol->ndim; ++d) nb *= (vol->n[d] + brick_of(d) - 1) / brick_of(d);
+            }
+            int chosen[3] = {cells[0], cells[1], cells[2]};
+            double best = fit(false) ? 0.93 * time_of() : 1e300;
+            for (int z = 0; z < n_z; ++z)
+                for (int y = 0; y < n_sizes; ++y)
+                    for (int x = 0; x < n_sizes; ++x) {
+                        cells[0] = sizes[x];
+                        cells[1] = sizes[y];
+                        cells[2] = sizes_z[z];
+                        if (cells[0] * cells[1] * cells[2] * G > 16 * 32) continue;
+                        for (int d = 0; d < vol->ndim; ++d) B[d] = brick_of(d);
+                        if (estimate(warps_of(), 0) >= best || !fit(false)) continue;   // without staging: a lower bound
+                        const double t = time_of();
+                        if (t < best) {
+                            best = t;
+                            for (int d = 0; d < 3; ++d) chosen[d] = cells[d];
+                        }
+                    }
+            for (int d = 0; d < 3; ++d) cells[d] = chosen[d];
         }
     }
+    if (fit(own_bricks)) return AC_OK;
     AC_FAIL(AC_ERR_ARG, "ac_evolve: staged region cannot fit the shared-memory budget; use smaller bricks");
+}
+
+// plan_evolve, or the plan of the owner's last launch when nothing that it depends on
+// has changed (a search over bricks costs about 20 us of host time).
+ac_status plan_with_memo(const ac_volume *vol, double stride_hint, double r_hint, const ac_evolve_params *p,
+                         PlanMemo &memo, Plan &pl)
+{
+    PlanKey key;
+    std::memset(&key, 0, sizeof(key));
+    key.dtype = vol->dtype;
+    key.ndim = vol->ndim;
+    for (int d = 0; d < 3; ++d) {
+        key.n[d] = vol->n[d];
+        key.sp[d] = vol->sp[d];
+        key.brick[d] = p->brick[d];
+    }
+    key.stride = stride_hint;
+    key.r = r_hint;
+    key.N = p->N;
+    key.T = p->T;
+    key.path = p->path;
+    key.lanes = p->lanes_per_contour;
+    key.comp = p->compensated;
+    key.warps = p->warps_per_block;
+    key.sampling = p->sampling;
+    key.dR = p->dR;
+    key.halo_factor = p->halo_factor;
+    if (memo.valid && std::memcmp(&memo.key, &key, sizeof(key)) == 0) {
+        pl = memo.plan;
+        return AC_OK;
+    }
+    memo.valid = false;
+    const ac_status s = plan_evolve(vol, stride_hint, r_hint, p, pl);
+    if (s != AC_OK) return s;
+    memo.key = key;
+    memo.plan = pl;
+    memo.valid = true;
+    return AC_OK;
 }
 
 CUtensorMapDataType tma_type(ac_dtype t)
@@ -916,7 +1036,7 @@ ac_status prepare_sets(ac_contours *const *sets, const ac_batch_item *items, int
         return AC_OK;
     }
     Plan &pl = pr.pl;
-    s = plan_evolve(v0, stride_hint, r_hint, p, pl);
+    s = plan_with_memo(v0, stride_hint, r_hint, p, sc.memo, pl);
     if (s != AC_OK) return s;
     pr.dtype = v0->dtype;
     pr.n_sets = n_sets;

@@ -79,7 +79,31 @@ struct HostBuf {
     template <typename T> T *as() const { return reinterpret_cast<T *>(p); }
 };
 
+// The launch layout of a set of contours (plan_evolve), and the last one of a handle
+// with everything it was made from.
+struct Plan {
+    int B[3], halo[3], ext[3];
+    int raw;        // staged region bytes
+    int quad_off;   // 2D: byte offset of the quads (0: none)
+    int smem;       // dynamic shared memory bytes
+    int G, warps;
+    bool brick, grid, comp, acc;
+};
+
+struct PlanKey {
+    int64_t n[3];
+    double stride, r;
+    float sp[3], dR, halo_factor;
+    int dtype, ndim, N, T, path, lanes, comp, warps, sampling, brick[3];
+};
+struct PlanMemo {
+    bool valid = false;
+    PlanKey key;
+    Plan plan;
+};
+
 struct Scratch {
+    PlanMemo memo;
     DevBuf keys, ranks, order, bin_table, desc, tmaps, active;       // evolve
     DevBuf flags, surv, ekeys, surv_sorted, pos, cellk, celli, cellk_s, celli_s, cell_start, stat, acc,
         cells, counters, cub;                                          // localize
