@@ -153,6 +153,23 @@ template <> __device__ __forceinline__ HQuad make_quad<HQuad>(float a, float b, 
     return HQuad{__floats2half2_rn(a, b), __floats2half2_rn(c, d)};
 }
 
+template <typename QT> __device__ __forceinline__ QT lds_quad(uint32_t a);
+template <> __device__ __forceinline__ float4 lds_quad<float4>(uint32_t a)
+{
+    float4 q;
+    asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "r"(a));
+    return q;
+}
+template <> __device__ __forceinline__ HQuad lds_quad<HQuad>(uint32_t a)
+{
+    uint32_t lo, hi;
+    asm("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(lo), "=r"(hi) : "r"(a));
+    HQuad q;
+    memcpy(&q.lo, &lo, 4);
+    memcpy(&q.hi, &hi, 4);
+    return q;
+}
+
 template <bool DIFF> __device__ __forceinline__ float quad_lerp(const float4 q, float f0, float f1)
 {
     const float2 v0 = make_float2(q.x, q.y);                       // (v00, v01)
@@ -161,18 +178,48 @@ template <bool DIFF> __device__ __forceinline__ float quad_lerp(const float4 q, 
     return fmaf(f1, a.y - a.x, a.x);
 }
 
+// Two 2D samples side by side (x: the first, y: the second): every gather below takes
+// pairs too, by default one sample after the other.
+template <typename Gather> __device__ __forceinline__ float2 at_each(const Gather &g, float2 x0, float2 x1)
+{
+    return make_float2(g.at(x0.x, x1.x, 0.0f), g.at(x0.y, x1.y, 0.0f));
+}
+
+// The index of a tap is formed in floating point: M0 is 2^23 plus the linear index of
+// the centre voxel, so that t0 + pitch * floor(x1) (+ ...) is 2^23 + the tap's linear
+// index, exactly (regions hold fewer than 2^18 elements), and its bits are an integer.
 template <typename QT, bool DIFF> struct QuadFast {
     const QT *Q;
     int qp;          // quads per row
-    float M[2];
+    float M[2];      // 2^23 + index of the centre voxel, per axis
     int nq;          // quads in the region (checked build)
     int32_t *st;     // status word (checked build)
+    uint32_t C;      // shared-memory address of Q, biases folded (modulo 2^32)
+    float M0, qpf;   // 2^23 + linear index of the centre voxel; quads per row
     __device__ __forceinline__ float at(float x0, float x1, float) const
     {
         int i0, i1;
         float2 fr;
         fast_axes2(make_float2(x0, x1), make_float2(M[0], M[1]), i0, i1, fr);
         return quad_lerp<DIFF>(quad_f(Q[checked(i1 * qp + i0, nq, st)]), fr.x, fr.y);
+    }
+    __device__ __forceinline__ float2 at2(float2 x0, float2 x1) const
+    {
+#ifdef AC_CHECKED
+        return at_each(*this, x0, x1);
+#else
+        const float2 t0 = __fadd2_rd(x0, dup2(M0)), t1 = __fadd2_rd(x1, dup2(M[1]));
+        const float2 l1 = sub2(t1, dup2(M[1]));
+        const float2 f0 = sub2(x0, sub2(t0, dup2(M0))), f1 = sub2(x1, l1);
+        const float2 i = fma2(l1, dup2(qpf), t0);
+        const float4 a = quad_f(lds_quad<QT>(C + (uint32_t)sizeof(QT) * __float_as_uint(i.x)));
+        const float4 b = quad_f(lds_quad<QT>(C + (uint32_t)sizeof(QT) * __float_as_uint(i.y)));
+        const float2 v0 = make_float2(a.x, b.x), v1 = make_float2(a.y, b.y);
+        const float2 e0 = make_float2(a.z, b.z), e1 = make_float2(a.w, b.w);
+        const float2 r0 = fma2(f0, DIFF ? e0 : sub2(e0, v0), v0);   // row y0 at x
+        const float2 r1 = fma2(f0, DIFF ? e1 : sub2(e1, v1), v1);   // row y1
+        return fma2(f1, sub2(r1, r0), r0);
+#endif
     }
 };
 
@@ -247,6 +294,7 @@ template <int DIM, typename T> struct RawFast {
         if (DIM == 3) fast_axis(x2, M[2], i2, f2);
         return interp<DIM, T>(p + i0 + i1 * py + i2 * pz, py, pz, fr.x, fr.y, f2, SmemLoad<T>{p, n, st});
     }
+    __device__ __forceinline__ float2 at2(float2 x0, float2 x1) const { return at_each(*this, x0, x1); }
 };
 
 // Raw taps through 32-bit shared-memory addresses (3D fast path; the bounds-checked
@@ -307,9 +355,9 @@ template <> __device__ __forceinline__ float lds_tap_next<float>(uint32_t a)
 }
 
 template <typename T> struct RawFast3S {
-    uint32_t C;      // folded base address (see above)
+    uint32_t C;          // folded base address (see above)
     uint32_t pyb, pzb;   // row and plane pitch, bytes
-    float M[3];
+    float M[3];          // 2^23 + index of the centre voxel, per axis
     __device__ __forceinline__ float at(float x0, float x1, float x2) const
     {
         constexpr float Z = TapBias<T>::value;
@@ -352,6 +400,7 @@ template <int DIM, typename T, bool QUAD> struct SmemClamp {
         const T *q = reinterpret_cast<const T *>(p) + (o[0] + b0) + (o[1] + b1) * py + (DIM == 3 ? (o[2] + b2) * pz : 0);
         return interp<DIM, T>(q, py, pz, f0, f1, f2, SmemLoad<T>{reinterpret_cast<const T *>(p), n, st});
     }
+    __device__ __forceinline__ float2 at2(float2 x0, float2 x1) const { return at_each(*this, x0, x1); }
 };
 
 // Clamped path from the row-pitched volume in global memory.
@@ -372,6 +421,7 @@ template <int DIM, typename T> struct GlobalClamp {
                      (DIM == 3 ? (int64_t)(ax[2].ci + b2) * pz : 0);
         return interp<DIM, T>(q, py, pz, f0, f1, f2, GlobalLoad<T>{p, n, st});
     }
+    __device__ __forceinline__ float2 at2(float2 x0, float2 x1) const { return at_each(*this, x0, x1); }
 };
 
 // ----------------------------------------------------------------- one sample
@@ -448,6 +498,53 @@ __device__ __forceinline__ void add_terms4(Acc &acc, const Terms &x, const Terms
     add_terms<DIM, COMP>(acc, sum4<DIM>(x, y, z, w));
 }
 
+// The same for two samples side by side, the products with the direction left to the
+// sums.
+struct Terms2 {
+    float2 J, JR;            // S I, dS/dR I
+    float2 g, d0, d1;        // -S' I, raw direction
+};
+
+__device__ __forceinline__ Terms2 pair_terms(const IterC<2> &ic, const EvolveArgs &a, float2 rv, float2 I, float2 d0,
+                                             float2 d1)
+{
+    const float2 t1 = fma2(rv, dup2(ic.A1), dup2(ic.B1)), t2 = fma2(rv, dup2(ic.A2), dup2(ic.B2));
+    const float2 r1 = make_float2(__saturatef(t1.x), __saturatef(t1.y));
+    const float2 r2 = make_float2(__saturatef(t2.x), __saturatef(t2.y));
+    const float2 S = sub2(fma2(dup2(2.0f), r1, dup2(-1.0f)), r2);
+    const float2 m1 = make_float2(r1.x == t1.x ? I.x : 0.0f, r1.y == t1.y ? I.y : 0.0f);
+    const float2 m2 = make_float2(r2.x == t2.x ? I.x : 0.0f, r2.y == t2.y ? I.y : 0.0f);
+    Terms2 o;
+    o.g = fma2(dup2(a.kr1), m1, mul2(dup2(a.kr2), m2));
+    o.JR = fma2(dup2(a.kR1), m1, mul2(dup2(a.kR2), m2));
+    o.J = make_float2(__fmul_rn(S.x, I.x), __fmul_rn(S.y, I.y));   // rounded before any sum
+    o.d0 = d0;
+    o.d1 = d1;
+    return o;
+}
+
+// The sum of the samples of a pair (x.x + x.y), and of two pairs ((p.x + q.x) +
+// (p.y + q.y)); of two products with the direction, the first is fused with the sum.
+__device__ __forceinline__ float dot_pair(float2 a, float2 b) { return __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)); }
+__device__ __forceinline__ Terms sum_pair(const Terms2 &p)
+{
+    Terms h;
+    h.a = make_float2(p.J.x + p.J.y, p.JR.x + p.JR.y);
+    h.b = make_float2(dot_pair(p.g, p.d0), dot_pair(p.g, p.d1));
+    h.c = 0.0f;
+    return h;
+}
+__device__ __forceinline__ Terms sum_pairs(const Terms2 &p, const Terms2 &q)
+{
+    const float2 J = add2(p.J, q.J), JR = add2(p.JR, q.JR);
+    const float2 c0 = fma2(p.g, p.d0, mul2(q.g, q.d0)), c1 = fma2(p.g, p.d1, mul2(q.g, q.d1));
+    Terms h;
+    h.a = make_float2(J.x + J.y, JR.x + JR.y);
+    h.b = make_float2(c0.x + c0.y, c1.x + c1.y);
+    h.c = 0.0f;
+    return h;
+}
+
 // All samples of one contour-iteration handled by this lane (lane `lig` of G).
 // The words of iteration n of contour k form the stream Philox(0, n, k, stream),
 // Philox(1, n, k, stream), ... (four words per block) and sample j takes words 2j
@@ -481,7 +578,7 @@ template <int DIM, bool ACC, typename Gather>
 __device__ __forceinline__ Terms sample3(const Gather &gat, const IterC<DIM> &ic, const EvolveArgs &a, uint32_t w0,
                                          uint32_t w1)
 {
-    const float b0 = __uint_as_float((w0 >> 11) | 0x4B000000u);
+    const float b0 = __uint_as_float(__funnelshift_r(w0, 0x258u, 11));   // (w0 >> 11) | 0x4B000000
     const float b1 = __uint_as_float((w1 & 0x1FFFFFu) | 0x4B000000u);
     const uint32_t u2 = __funnelshift_l(w1, w0, 10) & 0x1FFFFFu;
     const float2 ut = fma2(make_float2(b0, b1), dup2(4.76837158203125e-7f), dup2(-4.0f));   // (b - 2^23) 2^-21
@@ -509,64 +606,107 @@ __device__ __forceinline__ Terms sample2(const Gather &gat, const IterC<DIM> &ic
     return sample_terms<DIM>(ic, a, rv, gat.at(x.x, x.y, 0.0f), d0, d1, 0.0f);
 }
 
+// Two 2D samples at once: every floating-point step of both in one packed instruction,
+// the pair (first, second) in one register pair from the words to the sums.  2D is
+// bound by instruction issue and the FMA pipes together; packing x with y within a
+// sample left the z-less steps (weights, sums, interpolation along y) scalar and paid
+// moves to build the pairs.  2048^2 u8, 10 iterations: 526 -> 494 us (79 -> 70
+// instructions a sample).  In 3D the same change saves 8 % of the instructions but is 4 %
+// slower: a packed operation holds both FMA pipes, and the heavy one, which also has
+// the generator's wide multiplies, goes from 53 to 65 % busy, so 3D keeps its scalar half.
+template <typename Gather>
+__device__ __forceinline__ Terms2 sample2_pair(const Gather &gat, const IterC<2> &ic, const EvolveArgs &a, uint32_t vr,
+                                               uint32_t va, uint32_t wr, uint32_t wa)
+{
+    const float2 rv = make_float2(sqrt_approx(top24(vr)), sqrt_approx(top24(wr)));
+    constexpr float ANG = 6.283185307179586f / 16777216.0f;   // 2 pi / 2^24
+    const float2 ang = fma2(make_float2(top24(va), top24(wa)), dup2(ANG), dup2(-3.14159265358979323846f));
+    const float2 d0 = make_float2(cos_approx(ang.x), cos_approx(ang.y));
+    const float2 d1 = make_float2(sin_approx(ang.x), sin_approx(ang.y));
+    const float2 x0 = fma2(mul2(rv, dup2(ic.K[0])), d0, dup2(ic.ax[0].cf));
+    const float2 x1 = fma2(mul2(rv, dup2(ic.K[1])), d1, dup2(ic.ax[1].cf));
+    return pair_terms(ic, a, rv, gat.at2(x0, x1), d0, d1);
+}
+
 template <int DIM, int G, bool COMP, bool ACC, typename Gather>
 __device__ __forceinline__ void sample_contour(const Gather &gat, const IterC<DIM> &ic, const EvolveArgs &a,
                                                uint32_t n, uint32_t k, uint32_t stream, int lig, Acc &acc)
 {
+    // block m gives samples 2m and 2m + 1
+    auto block = [&](int m) { return philox4x32_10(make_uint4((uint32_t)m, n, k, stream), a.rk0, a.rk1); };
+    const int pairs = a.N >> 1;
+    int m = lig;
     if constexpr (DIM == 3) {
-        // block m gives samples 2m and 2m + 1; a lane takes blocks m and m + G (four
-        // samples, summed in two roundings before one compensated addition), then a
-        // leftover block, then an odd N's last sample
-        const int pairs = a.N >> 1;
-        int m = lig;
+        // a lane takes blocks m and m + G (four samples, summed in two roundings before
+        // one compensated addition), then a leftover block, then an odd N's last sample
 #pragma unroll 1
         for (; m + G < pairs; m += 2 * G) {
-            const uint4 A = philox4x32_10(make_uint4((uint32_t)m, n, k, stream), a.rk0, a.rk1);
-            const uint4 B = philox4x32_10(make_uint4((uint32_t)(m + G), n, k, stream), a.rk0, a.rk1);
+            const uint4 A = block(m), B = block(m + G);
             add_terms4<DIM, COMP>(acc, sample3<DIM, ACC>(gat, ic, a, A.x, A.y), sample3<DIM, ACC>(gat, ic, a, A.z, A.w),
                                   sample3<DIM, ACC>(gat, ic, a, B.x, B.y), sample3<DIM, ACC>(gat, ic, a, B.z, B.w));
         }
         if (m < pairs) {
-            const uint4 A = philox4x32_10(make_uint4((uint32_t)m, n, k, stream), a.rk0, a.rk1);
+            const uint4 A = block(m);
             add_terms<DIM, COMP>(acc, sample3<DIM, ACC>(gat, ic, a, A.x, A.y), sample3<DIM, ACC>(gat, ic, a, A.z, A.w));
         }
         if ((a.N & 1) && lig == pairs % G) {
-            const uint4 A = philox4x32_10(make_uint4((uint32_t)pairs, n, k, stream), a.rk0, a.rk1);
+            const uint4 A = block(pairs);
             add_terms<DIM, COMP>(acc, sample3<DIM, ACC>(gat, ic, a, A.x, A.y));
         }
-    } else {
+    } else if constexpr (ACC) {
         // the two samples of a Philox block form a pair; four blocks of a lane (m,
         // m + G, m + 2G, m + 3G) are summed pairwise in three roundings before one
         // compensated addition, then two blocks, then a leftover block and an odd
         // N's last sample
-        const int pairs = a.N >> 1;
-        int m = lig;
 #pragma unroll 1
         for (; m + 3 * G < pairs; m += 4 * G) {
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)m, n, k, stream), a.rk0, a.rk1);
-            const uint4 u = philox4x32_10(make_uint4((uint32_t)(m + G), n, k, stream), a.rk0, a.rk1);
-            const Terms h = sum4<DIM>(sample2<DIM, ACC>(gat, ic, a, w.x, w.y), sample2<DIM, ACC>(gat, ic, a, w.z, w.w),
-                                      sample2<DIM, ACC>(gat, ic, a, u.x, u.y), sample2<DIM, ACC>(gat, ic, a, u.z, u.w));
-            const uint4 w2 = philox4x32_10(make_uint4((uint32_t)(m + 2 * G), n, k, stream), a.rk0, a.rk1);
-            const uint4 u2 = philox4x32_10(make_uint4((uint32_t)(m + 3 * G), n, k, stream), a.rk0, a.rk1);
-            const Terms q = sum4<DIM>(sample2<DIM, ACC>(gat, ic, a, w2.x, w2.y), sample2<DIM, ACC>(gat, ic, a, w2.z, w2.w),
-                                      sample2<DIM, ACC>(gat, ic, a, u2.x, u2.y), sample2<DIM, ACC>(gat, ic, a, u2.z, u2.w));
+            const uint4 w = block(m);
+            const uint4 u = block(m + G);
+            const Terms h = sum4<DIM>(sample2<DIM, true>(gat, ic, a, w.x, w.y), sample2<DIM, true>(gat, ic, a, w.z, w.w),
+                                      sample2<DIM, true>(gat, ic, a, u.x, u.y), sample2<DIM, true>(gat, ic, a, u.z, u.w));
+            const uint4 w2 = block(m + 2 * G);
+            const uint4 u2 = block(m + 3 * G);
+            const Terms q = sum4<DIM>(sample2<DIM, true>(gat, ic, a, w2.x, w2.y), sample2<DIM, true>(gat, ic, a, w2.z, w2.w),
+                                      sample2<DIM, true>(gat, ic, a, u2.x, u2.y), sample2<DIM, true>(gat, ic, a, u2.z, u2.w));
             add_terms<DIM, COMP>(acc, h, q);
         }
 #pragma unroll 1
         for (; m + G < pairs; m += 2 * G) {
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)m, n, k, stream), a.rk0, a.rk1);
-            const uint4 u = philox4x32_10(make_uint4((uint32_t)(m + G), n, k, stream), a.rk0, a.rk1);
-            add_terms4<DIM, COMP>(acc, sample2<DIM, ACC>(gat, ic, a, w.x, w.y), sample2<DIM, ACC>(gat, ic, a, w.z, w.w),
-                                  sample2<DIM, ACC>(gat, ic, a, u.x, u.y), sample2<DIM, ACC>(gat, ic, a, u.z, u.w));
+            const uint4 w = block(m);
+            const uint4 u = block(m + G);
+            add_terms4<DIM, COMP>(acc, sample2<DIM, true>(gat, ic, a, w.x, w.y), sample2<DIM, true>(gat, ic, a, w.z, w.w),
+                                  sample2<DIM, true>(gat, ic, a, u.x, u.y), sample2<DIM, true>(gat, ic, a, u.z, u.w));
         }
         if (m < pairs) {
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)m, n, k, stream), a.rk0, a.rk1);
-            add_terms<DIM, COMP>(acc, sample2<DIM, ACC>(gat, ic, a, w.x, w.y), sample2<DIM, ACC>(gat, ic, a, w.z, w.w));
+            const uint4 w = block(m);
+            add_terms<DIM, COMP>(acc, sample2<DIM, true>(gat, ic, a, w.x, w.y), sample2<DIM, true>(gat, ic, a, w.z, w.w));
         }
         if ((a.N & 1) && lig == pairs % G) {
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)pairs, n, k, stream), a.rk0, a.rk1);
-            add_terms<DIM, COMP>(acc, sample2<DIM, ACC>(gat, ic, a, w.x, w.y));
+            const uint4 w = block(pairs);
+            add_terms<DIM, COMP>(acc, sample2<DIM, true>(gat, ic, a, w.x, w.y));
+        }
+    } else {
+        // the same with two samples side by side in packed instructions: the first samples
+        // of blocks m and m + G, then their second samples
+        auto two = [&](const uint4 &A, const uint4 &B) {
+            return sum_pairs(sample2_pair(gat, ic, a, A.x, A.y, B.x, B.y),
+                                  sample2_pair(gat, ic, a, A.z, A.w, B.z, B.w));
+        };
+#pragma unroll 1
+        for (; m + 3 * G < pairs; m += 4 * G) {
+            const Terms h = two(block(m), block(m + G));
+            const Terms q = two(block(m + 2 * G), block(m + 3 * G));
+            add_terms<DIM, COMP>(acc, h, q);
+        }
+#pragma unroll 1
+        for (; m + G < pairs; m += 2 * G) add_terms<DIM, COMP>(acc, two(block(m), block(m + G)));
+        if (m < pairs) {
+            const uint4 A = block(m);
+            add_terms<DIM, COMP>(acc, sum_pair(sample2_pair(gat, ic, a, A.x, A.y, A.z, A.w)));
+        }
+        if ((a.N & 1) && lig == pairs % G) {
+            const uint4 A = block(pairs);
+            add_terms<DIM, COMP>(acc, sample2<DIM, ACC>(gat, ic, a, A.x, A.y));
         }
     }
 }
@@ -816,8 +956,9 @@ __global__ void __maxnreg__(DIM == 2 ? 96 : 128) evolve_brick_kernel(const __gri
     }
 
     const int py = a.ext[0], pz = a.ext[0] * a.ext[1];
-    // base of the 32-bit tap addresses of the 3D fast path, biases folded (modulo 2^32)
+    // base of the 32-bit tap and quad addresses of the fast paths, biases folded (modulo 2^32)
     const uint32_t raw_C = smem_u32(smem_raw) - (uint32_t)sizeof(T) * 0x4B000000u * (uint32_t)(1 + py + pz);
+    const uint32_t quad_C = smem_u32(Q) - (uint32_t)sizeof(QT) * 0x4B000000u;
     // the staged region's first and last usable tap per axis (within the volume)
     float fr_lo[3], fr_hi[3];
 #pragma unroll
@@ -909,7 +1050,8 @@ __global__ void __maxnreg__(DIM == 2 ? 96 : 128) evolve_brick_kernel(const __gri
             if (use_fast) {
                 const float M[3] = {8388608.0f + (float)o[0], 8388608.0f + (float)o[1], 8388608.0f + (float)o[2]};
                 if (quad) {
-                    QuadFast<QT, QuadOf<T>::diff> gat{Q, qp, {M[0], M[1]}, nquads, V.status};
+                    QuadFast<QT, QuadOf<T>::diff> gat{Q, qp, {M[0], M[1]}, nquads, V.status, quad_C,
+                                                      8388608.0f + (float)(o[0] + o[1] * qp), (float)qp};
                     s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
                 } else {
 #ifndef AC_CHECKED
