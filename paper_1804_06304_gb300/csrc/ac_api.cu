@@ -705,10 +705,9 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
                 raw *= ext;
             }
             int64_t quad_off = 0, total = raw;
-            if (vol->ndim == 2) {   // quads after the raw region: 4 halves (uint8, binary16) or float4
-                const int qbytes = (vol->dtype == AC_U8 || vol->dtype == AC_F16) ? 8 : 16;
+            if (vol->ndim == 2 && vol->dtype != AC_F32) {   // 8-byte quads after the raw region
                 quad_off = (raw + 127) / 128 * 128;
-                total = quad_off + (int64_t)(pl.ext[0] - 1) * (pl.ext[1] - 1) * qbytes;
+                total = quad_off + (int64_t)(pl.ext[0] - 1) * (pl.ext[1] - 1) * 8;
             }
             if (fits_box && total <= budget) {
                 pl.raw = (int)raw;
@@ -785,7 +784,7 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
                 const double busy = std::min(lattice / nb / per_warp, (double)warps);   // warps at work, on average
                 const double most = std::min((double)warps, std::ceil(full / per_warp));
                 const double passes = std::ceil(full / per_warp / warps);
-                const double quads = vol->ndim == 2 ? smem / (vol->es == 1 ? 9.0 : 20.0) / (warps * 32) * 1000.0 : 0.0;
+                const double quads = vol->ndim == 2 && vol->dtype != AC_F32 ? smem / (8.0 + vol->es) / (warps * 32) * 1000.0 : 0.0;
                 const double stage = 3000.0 + smem / 14.4 + quads;
                 const double k = nb / 152.0, whole = std::floor(k / r);
                 double t = whole * (stage + instr * passes * f(r * busy / 4));

@@ -9,6 +9,8 @@
 // the voxels come from; the paths therefore give bit-identical results.
 #pragma once
 
+#include <type_traits>
+
 #include "ac_internal.cuh"
 
 namespace ac {
@@ -114,67 +116,80 @@ __device__ __forceinline__ void fast_axes2(float2 x, float2 M, int &i0, int &i1,
     i1 = (int)__float_as_uint(t.y) - 0x4B000000;
 }
 
-// 2D region as quads: one shared-memory load feeds a bilinear sample.  With
-// `diff`, a quad holds (v00, v01, v10 - v00, v11 - v01), the values of the two rows
-// and the x-differences the interpolation needs (computed once per quad in FP32, as
-// the sample would), so both rows are interpolated in one packed operation; else
-// (v00, v01, v10, v11).  Four halves (8 bytes) for uint8 voxels (values and
-// differences are integers below 2^9, exact in half precision) and binary16 voxels
-// (values only: their differences need not be representable), float4 otherwise.
-struct HQuad {
+// 2D region as quads of 8 bytes: one shared-memory load feeds a bilinear sample.
+// uint8 voxels: halves (v00, v01, v10 - v00, v11 - v01), the values of the two rows and
+// the x-differences the interpolation needs (integers below 2^9, exact in half
+// precision), so both rows are interpolated without a subtraction (`diff`); binary16
+// voxels: (v00, v01, v10, v11), because their differences need not be representable;
+// uint16 voxels: (v00, v01, v10, v11) as stored.  float voxels have no quads: at 16
+// bytes each they would leave room for one CTA of 10 warps per SM, and four 4-byte
+// loads are cheaper than that (2048^2, 10 iterations: 643 -> 465 us; uint16 with 8
+// instead of 16 bytes 647 -> 485 us).  A warp fills a row of quads at a time, without the
+// division that a flat index needs (uint8: 494 -> 477 us).
+struct __align__(8) HQuad {
     __half2 lo, hi;
 };
+struct __align__(8) UQuad {
+    uint32_t lo, hi;   // v00 | v01 << 16, v10 | v11 << 16
+};
 template <typename T> struct QuadOf {
-    using type = float4;
-    static constexpr bool diff = true;
+    using type = HQuad;
+    static constexpr bool quads = false, diff = false;
 };
 template <> struct QuadOf<uint8_t> {
     using type = HQuad;
-    static constexpr bool diff = true;
+    static constexpr bool quads = true, diff = true;
 };
 template <> struct QuadOf<__half> {
     using type = HQuad;
-    static constexpr bool diff = false;
+    static constexpr bool quads = true, diff = false;
+};
+template <> struct QuadOf<uint16_t> {
+    using type = UQuad;
+    static constexpr bool quads = true, diff = false;
 };
 
-__device__ __forceinline__ float4 quad_f(const float4 &q) { return q; }
+// The four numbers of a quad; `bias` is what the values carry on top (the differences
+// of two of them do not).
 __device__ __forceinline__ float4 quad_f(const HQuad &q)
 {
     const float2 a = __half22float2(q.lo), b = __half22float2(q.hi);
     return make_float4(a.x, a.y, b.x, b.y);
 }
-template <typename QT> __device__ __forceinline__ QT make_quad(float a, float b, float c, float d);
-template <> __device__ __forceinline__ float4 make_quad<float4>(float a, float b, float c, float d)
+__device__ __forceinline__ float4 quad_f(const UQuad &q)
 {
-    return make_float4(a, b, c, d);
+    // 0x4B00 above the low or the high half: 2^23 + v
+    return make_float4(__uint_as_float(__byte_perm(q.lo, 0x4B00u, 0x5410)), __uint_as_float(__byte_perm(q.lo, 0x4B00u, 0x5432)),
+                       __uint_as_float(__byte_perm(q.hi, 0x4B00u, 0x5410)), __uint_as_float(__byte_perm(q.hi, 0x4B00u, 0x5432)));
 }
-template <> __device__ __forceinline__ HQuad make_quad<HQuad>(float a, float b, float c, float d)
+template <typename QT> struct QuadBias {
+    static constexpr float value = 0.0f;
+};
+template <> struct QuadBias<UQuad> {
+    static constexpr float value = 8388608.0f;
+};
+__device__ __forceinline__ void make_quad(HQuad &q, float a, float b, float c, float d)
 {
-    return HQuad{__floats2half2_rn(a, b), __floats2half2_rn(c, d)};
+    q = HQuad{__floats2half2_rn(a, b), __floats2half2_rn(c, d)};
 }
 
-template <typename QT> __device__ __forceinline__ QT lds_quad(uint32_t a);
-template <> __device__ __forceinline__ float4 lds_quad<float4>(uint32_t a)
-{
-    float4 q;
-    asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "r"(a));
-    return q;
-}
-template <> __device__ __forceinline__ HQuad lds_quad<HQuad>(uint32_t a)
+template <typename QT> __device__ __forceinline__ QT lds_quad(uint32_t a)
 {
     uint32_t lo, hi;
     asm("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(lo), "=r"(hi) : "r"(a));
-    HQuad q;
+    QT q;
     memcpy(&q.lo, &lo, 4);
     memcpy(&q.hi, &hi, 4);
     return q;
 }
 
-template <bool DIFF> __device__ __forceinline__ float quad_lerp(const float4 q, float f0, float f1)
+template <typename QT, bool DIFF> __device__ __forceinline__ float quad_lerp(const QT &quad, float f0, float f1)
 {
-    const float2 v0 = make_float2(q.x, q.y);                       // (v00, v01)
-    const float2 d = DIFF ? make_float2(q.z, q.w) : sub2(make_float2(q.z, q.w), v0);
-    const float2 a = fma2(dup2(f0), d, v0);                        // the two rows at x
+    constexpr float Z = QuadBias<QT>::value;
+    const float4 q = quad_f(quad);
+    const float2 v = make_float2(q.x, q.y);                        // (v00, v01)
+    const float2 d = DIFF ? make_float2(q.z, q.w) : sub2(make_float2(q.z, q.w), v);
+    const float2 a = fma2(dup2(f0), d, Z != 0.0f ? sub2(v, dup2(Z)) : v);   // the two rows at x
     return fmaf(f1, a.y - a.x, a.x);
 }
 
@@ -186,8 +201,20 @@ template <typename Gather> __device__ __forceinline__ float2 at_each(const Gathe
 }
 
 // The index of a tap is formed in floating point: M0 is 2^23 plus the linear index of
-// the centre voxel, so that t0 + pitch * floor(x1) (+ ...) is 2^23 + the tap's linear
-// index, exactly (regions hold fewer than 2^18 elements), and its bits are an integer.
+// the centre voxel, so that t0 + pitch * floor(x1) is 2^23 + the tap's linear index,
+// exactly (regions hold fewer than 2^18 elements), and its bits are an integer.
+struct FastIndex2 {
+    float2 i, f0, f1;   // 2^23 + index, fractions
+    __device__ __forceinline__ FastIndex2(float2 x0, float2 x1, float M0, float M1, float pitch)
+    {
+        const float2 t0 = __fadd2_rd(x0, dup2(M0)), t1 = __fadd2_rd(x1, dup2(M1));
+        const float2 l1 = sub2(t1, dup2(M1));
+        f0 = sub2(x0, sub2(t0, dup2(M0)));
+        f1 = sub2(x1, l1);
+        i = fma2(l1, dup2(pitch), t0);
+    }
+};
+
 template <typename QT, bool DIFF> struct QuadFast {
     const QT *Q;
     int qp;          // quads per row
@@ -195,30 +222,28 @@ template <typename QT, bool DIFF> struct QuadFast {
     int nq;          // quads in the region (checked build)
     int32_t *st;     // status word (checked build)
     uint32_t C;      // shared-memory address of Q, biases folded (modulo 2^32)
-    float M0, qpf;   // 2^23 + linear index of the centre voxel; quads per row
+    float M0, pitch; // 2^23 + linear index of the centre voxel; quads per row
     __device__ __forceinline__ float at(float x0, float x1, float) const
     {
         int i0, i1;
         float2 fr;
         fast_axes2(make_float2(x0, x1), make_float2(M[0], M[1]), i0, i1, fr);
-        return quad_lerp<DIFF>(quad_f(Q[checked(i1 * qp + i0, nq, st)]), fr.x, fr.y);
+        return quad_lerp<QT, DIFF>(Q[checked(i1 * qp + i0, nq, st)], fr.x, fr.y);
     }
     __device__ __forceinline__ float2 at2(float2 x0, float2 x1) const
     {
 #ifdef AC_CHECKED
         return at_each(*this, x0, x1);
 #else
-        const float2 t0 = __fadd2_rd(x0, dup2(M0)), t1 = __fadd2_rd(x1, dup2(M[1]));
-        const float2 l1 = sub2(t1, dup2(M[1]));
-        const float2 f0 = sub2(x0, sub2(t0, dup2(M0))), f1 = sub2(x1, l1);
-        const float2 i = fma2(l1, dup2(qpf), t0);
-        const float4 a = quad_f(lds_quad<QT>(C + (uint32_t)sizeof(QT) * __float_as_uint(i.x)));
-        const float4 b = quad_f(lds_quad<QT>(C + (uint32_t)sizeof(QT) * __float_as_uint(i.y)));
+        constexpr float Z = QuadBias<QT>::value;
+        const FastIndex2 t(x0, x1, M0, M[1], pitch);
+        const float4 a = quad_f(lds_quad<QT>(C + (uint32_t)sizeof(QT) * __float_as_uint(t.i.x)));
+        const float4 b = quad_f(lds_quad<QT>(C + (uint32_t)sizeof(QT) * __float_as_uint(t.i.y)));
         const float2 v0 = make_float2(a.x, b.x), v1 = make_float2(a.y, b.y);
         const float2 e0 = make_float2(a.z, b.z), e1 = make_float2(a.w, b.w);
-        const float2 r0 = fma2(f0, DIFF ? e0 : sub2(e0, v0), v0);   // row y0 at x
-        const float2 r1 = fma2(f0, DIFF ? e1 : sub2(e1, v1), v1);   // row y1
-        return fma2(f1, sub2(r1, r0), r0);
+        const float2 r0 = fma2(t.f0, DIFF ? e0 : sub2(e0, v0), Z != 0.0f ? sub2(v0, dup2(Z)) : v0);   // row y0 at x
+        const float2 r1 = fma2(t.f0, DIFF ? e1 : sub2(e1, v1), Z != 0.0f ? sub2(v1, dup2(Z)) : v1);   // row y1
+        return fma2(t.f1, sub2(r1, r0), r0);
 #endif
     }
 };
@@ -377,6 +402,32 @@ template <typename T> struct RawFast3S {
     }
 };
 
+// The 2D fast path without quads: four taps a sample, two samples at once.
+template <typename T> struct RawFast2S {
+    RawFast<2, T> one;
+    uint32_t C, pyb;     // address of the region, biases folded (modulo 2^32); row pitch, bytes
+    float M0, pitch;     // 2^23 + linear index of the centre voxel; elements per row
+    __device__ __forceinline__ float at(float x0, float x1, float x2) const { return one.at(x0, x1, x2); }
+    __device__ __forceinline__ float2 at2(float2 x0, float2 x1) const
+    {
+#ifdef AC_CHECKED
+        return at_each(one, x0, x1);
+#else
+        constexpr float Z = TapBias<T>::value;
+        const FastIndex2 t(x0, x1, M0, one.M[1], pitch);
+        const uint32_t a = C + (uint32_t)sizeof(T) * __float_as_uint(t.i.x);
+        const uint32_t b = C + (uint32_t)sizeof(T) * __float_as_uint(t.i.y);
+        auto row = [&](uint32_t p, uint32_t q) {
+            const float2 lo = make_float2(lds_tap<T>(p), lds_tap<T>(q));
+            const float2 hi = make_float2(lds_tap_next<T>(p), lds_tap_next<T>(q));
+            return fma2(t.f0, sub2(hi, lo), Z != 0.0f ? sub2(lo, dup2(Z)) : lo);
+        };
+        const float2 r0 = row(a, b), r1 = row(a + pyb, b + pyb);
+        return fma2(t.f1, sub2(r1, r0), r0);
+#endif
+    }
+};
+
 // Clamped path in shared memory (quads in 2D, raw voxels otherwise).
 template <int DIM, typename T, bool QUAD> struct SmemClamp {
     const void *p;
@@ -395,7 +446,7 @@ template <int DIM, typename T, bool QUAD> struct SmemClamp {
         if (QUAD) {
             using QT = typename QuadOf<T>::type;
             const int64_t qi = checked((int64_t)(o[1] + b1) * py + (o[0] + b0), n, st);
-            return quad_lerp<QuadOf<T>::diff>(quad_f(reinterpret_cast<const QT *>(p)[qi]), f0, f1);
+            return quad_lerp<QT, QuadOf<T>::diff>(reinterpret_cast<const QT *>(p)[qi], f0, f1);
         }
         const T *q = reinterpret_cast<const T *>(p) + (o[0] + b0) + (o[1] + b1) * py + (DIM == 3 ? (o[2] + b2) * pz : 0);
         return interp<DIM, T>(q, py, pz, f0, f1, f2, SmemLoad<T>{reinterpret_cast<const T *>(p), n, st});
@@ -940,24 +991,30 @@ __global__ void __maxnreg__(DIM == 2 ? 96 : 128) evolve_brick_kernel(const __gri
     // each thread observes the completed phase itself (at once) before reading the region
     mbar_wait_bounded(&mbar, 0, TMA_DRAIN_POLLS);
     const T *reg = reinterpret_cast<const T *>(smem_raw);
-    const bool quad = DIM == 2 && a.quad_off > 0;
+    constexpr bool quad = DIM == 2 && QuadOf<T>::quads;
     QT *Q = reinterpret_cast<QT *>(smem_raw + a.quad_off);
     const int qp = a.ext[0] - 1;
-    if (quad) {
-        const int nq = qp * (a.ext[1] - 1);
-        for (int i = threadIdx.x; i < nq; i += blockDim.x) {
-            const int y = i / qp, x = i - y * qp;
-            const T *r = reg + y * a.ext[0] + x;
-            const float v00 = to_f<T>(r[0]), v10 = to_f<T>(r[1]);
-            const float v01 = to_f<T>(r[a.ext[0]]), v11 = to_f<T>(r[a.ext[0] + 1]);
-            Q[i] = QuadOf<T>::diff ? make_quad<QT>(v00, v01, v10 - v00, v11 - v01) : make_quad<QT>(v00, v01, v10, v11);
+    if constexpr (quad) {   // a warp per row
+        for (int y = threadIdx.x >> 5; y < a.ext[1] - 1; y += blockDim.x >> 5) {
+            const T *r0 = reg + y * a.ext[0], *r1 = r0 + a.ext[0];
+            QT *row = Q + y * qp;
+#pragma unroll 4
+            for (int x = threadIdx.x & 31; x < qp; x += 32) {
+                if constexpr (std::is_same<QT, UQuad>::value) {
+                    row[x] = UQuad{r0[x] | (uint32_t)r1[x] << 16, r0[x + 1] | (uint32_t)r1[x + 1] << 16};
+                } else {
+                    const float v00 = to_f<T>(r0[x]), v10 = to_f<T>(r0[x + 1]);
+                    const float v01 = to_f<T>(r1[x]), v11 = to_f<T>(r1[x + 1]);
+                    make_quad(row[x], v00, v01, QuadOf<T>::diff ? v10 - v00 : v10, QuadOf<T>::diff ? v11 - v01 : v11);
+                }
+            }
         }
         __syncthreads();
     }
 
     const int py = a.ext[0], pz = a.ext[0] * a.ext[1];
-    // base of the 32-bit tap and quad addresses of the fast paths, biases folded (modulo 2^32)
-    const uint32_t raw_C = smem_u32(smem_raw) - (uint32_t)sizeof(T) * 0x4B000000u * (uint32_t)(1 + py + pz);
+    // bases of the 32-bit addresses of the fast paths, biases folded (modulo 2^32)
+    const uint32_t raw_C = smem_u32(smem_raw) - (uint32_t)sizeof(T) * 0x4B000000u * (uint32_t)(DIM == 3 ? 1 + py + pz : 1);
     const uint32_t quad_C = smem_u32(Q) - (uint32_t)sizeof(QT) * 0x4B000000u;
     // the staged region's first and last usable tap per axis (within the volume)
     float fr_lo[3], fr_hi[3];
@@ -1049,35 +1106,29 @@ __global__ void __maxnreg__(DIM == 2 ? 96 : 128) evolve_brick_kernel(const __gri
             n_global += use_smem ? 0u : 1u;
             if (use_fast) {
                 const float M[3] = {8388608.0f + (float)o[0], 8388608.0f + (float)o[1], 8388608.0f + (float)o[2]};
-                if (quad) {
+                if constexpr (quad) {
                     QuadFast<QT, QuadOf<T>::diff> gat{Q, qp, {M[0], M[1]}, nquads, V.status, quad_C,
                                                       8388608.0f + (float)(o[0] + o[1] * qp), (float)qp};
                     s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
+                } else if constexpr (DIM == 2) {
+                    RawFast2S<T> gat{{reg, py, pz, {M[0], M[1], M[2]}, nraw, V.status}, raw_C, (uint32_t)(sizeof(T) * py),
+                                     8388608.0f + (float)(o[0] + o[1] * py), (float)py};
+                    s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
                 } else {
 #ifndef AC_CHECKED
-                    if constexpr (DIM == 3) {   // 32-bit shared addresses, biases folded into raw_C
-                        RawFast3S<T> gat{raw_C, (uint32_t)(sizeof(T) * py), (uint32_t)(sizeof(T) * pz),
-                                         {M[0], M[1], M[2]}};
-                        s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig,
-                                                            mask);
-                    } else
+                    // 32-bit shared addresses, biases folded into raw_C
+                    RawFast3S<T> gat{raw_C, (uint32_t)(sizeof(T) * py), (uint32_t)(sizeof(T) * pz), {M[0], M[1], M[2]}};
+#else
+                    RawFast<DIM, T> gat{reg, py, pz, {M[0], M[1], M[2]}, nraw, V.status};
 #endif
-                    {
-                        RawFast<DIM, T> gat{reg, py, pz, {M[0], M[1], M[2]}, nraw, V.status};
-                        s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig,
-                                                            mask);
-                    }
+                    s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
                 }
             } else if (use_smem) {
-                if (quad) {
-                    SmemClamp<DIM, T, true> gat{Q, qp, 0, {ic.ax[0], ic.ax[1], ic.ax[2]}, {o[0], o[1], o[2]},
-                                                nquads, V.status};
-                    s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
-                } else {
-                    SmemClamp<DIM, T, false> gat{reg, py, pz, {ic.ax[0], ic.ax[1], ic.ax[2]}, {o[0], o[1], o[2]},
-                                                 nraw, V.status};
-                    s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
-                }
+                const int pitch = quad ? qp : py;
+                SmemClamp<DIM, T, quad> gat{quad ? (const void *)Q : (const void *)reg, pitch, quad ? 0 : pz,
+                                            {ic.ax[0], ic.ax[1], ic.ax[2]}, {o[0], o[1], o[2]},
+                                            quad ? (int64_t)nquads : nraw, V.status};
+                s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
             } else {
                 GlobalClamp<DIM, T> gat{reinterpret_cast<const T *>(V.data), V.pitch_y, V.pitch_z,
                                         {ic.ax[0], ic.ax[1], ic.ax[2]}, V.pitch_z * V.n[2], V.status};
