@@ -351,8 +351,8 @@ ac_status ac_localize(ac_contours *ctr, const ac_localize_params *params, ac_cel
  * writes up to caps[i] cells to out_host[i] (host memory, caller-owned) and its
  * total count to n_out[i]; the cells of each set are those ac_localize gives for
  * it alone.  The sets' work is queued phase by phase on one stream, so the call
- * synchronizes the stream four times (plus once per further eight competition
- * rounds) whatever n_sets is, instead of several times per set.  The first set's
+ * synchronizes the stream two or three times (plus once per further competition
+ * round) whatever n_sets is, instead of several times per set.  The first set's
  * handle holds the call's temporary buffers (sized for the whole batch).  Errors:
  * AC_ERR_ARG (NULL arrays, a NULL or repeated set, a negative cap, a NaN E0, more
  * than 65535 sets or 2^31 - 1 contours in one call), and the first failing set's

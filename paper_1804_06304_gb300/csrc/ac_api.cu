@@ -26,10 +26,8 @@ void count_launch(int64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed
 void Scratch::release_all()
 {
     DevBuf *all[] = {&keys, &ranks, &order, &bin_table, &cub, &desc, &tmaps, &active, &flags, &surv, &ekeys, &surv_sorted,
-                     &pos, &cellk, &celli, &cellk_s, &celli_s, &cell_start, &stat, &acc, &cells, &counters};
+                     &pos, &cellk, &celli, &list, &list_pos, &cell_start, &stat, &acc, &cells, &counters, &lsets};
     for (DevBuf *b : all) b->release();
-    lsets.release();
-    und.release();
     hcount.release();
     hcells.release();
     hsets.release();

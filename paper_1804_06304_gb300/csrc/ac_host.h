@@ -105,9 +105,8 @@ struct PlanMemo {
 struct Scratch {
     PlanMemo memo;
     DevBuf keys, ranks, order, bin_table, desc, tmaps, active;       // evolve
-    DevBuf flags, surv, ekeys, surv_sorted, pos, cellk, celli, cellk_s, celli_s, cell_start, stat, acc,
-        cells, counters, cub;                                          // localize
-    DevBuf lsets, und;                                                 // localize: set descriptors, open counts
+    DevBuf flags, surv, ekeys, surv_sorted, pos, cellk, celli, list, list_pos, cell_start, stat, acc,
+        cells, counters, cub, lsets;                                   // localize
     HostBuf hcount, hcells, hsets;                                     // localize: read back / uploaded
     void release_all();
 };
@@ -202,8 +201,8 @@ ac_status plan_set_trace(ac_plan *plan, int set, const ac_trace *trace);
 
 // localization (ac_localize.cu) of n distinct sets in one pass on one stream,
 // each with its own threshold, host output and cap; the first set's scratch holds
-// the batch's buffers.  The whole batch synchronizes the stream four times (plus
-// once per further eight competition rounds).  Returns an ac_status (the first
+// the batch's buffers.  The whole batch synchronizes the stream two or three times
+// (plus once per further competition round).  Returns an ac_status (the first
 // failing set's) and sets the message.
 ac_status localize_many(ac_contours *const *sets, const float *E0, ac_cell *const *out_host, const int64_t *cap,
                         int64_t *n_out, int n, cudaStream_t st);

@@ -8,15 +8,17 @@
 // every overlapping contour of higher priority is rejected, and rejected as soon
 // as one of them is accepted (the lexicographically first maximal independent
 // set).  Neighbours are found through a uniform grid of cell size
-// rho max(R), built with a sort.
+// rho max(R), built by counting.  Within a round a contour whose higher-priority
+// neighbours are still open looks again a bounded number of times, so one round settles
+// nearly everything.
 //
 // Any number of contour sets is localized in one pass: their contours are
 // indexed one after another (set-major), the cull and the selection of survivors
 // run once over all of them, one sort by (set, E, k) gives every set's priority
 // order, every set has its own grid, placed one after another in one cell index
-// space sorted once, and each round decides survivors of all sets at once.  A
-// batch costs the same few launches and four stream synchronisations whatever
-// the number of sets.
+// space, and each round decides survivors of all sets at once.  A batch costs the same
+// few launches and two stream synchronisations (three when many survive) whatever the
+// number of sets.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -66,8 +68,8 @@ struct LocSet {
 };
 
 // Per-set counters, CNT_N int32 per set in one device array (and its page-locked
-// copy); two batch totals follow them.
-enum { CNT_SURV, CNT_MAXR, CNT_STATUS, CNT_ABASE, CNT_ACC, CNT_N };
+// copy); two batch totals follow them.  CNT_OPEN: survivors a round left undecided.
+enum { CNT_SURV, CNT_MAXR, CNT_STATUS, CNT_ABASE, CNT_ACC, CNT_OPEN, CNT_N };
 
 // the set holding batch position `i` of the index whose set offsets are `base`
 // (sets in increasing order of their offsets)
@@ -82,19 +84,17 @@ __device__ __forceinline__ int set_of(const LocSet *sets, int nsets, int64_t i)
     return lo;
 }
 
-__global__ void status_kernel(const LocSet *sets, int nsets, int32_t *cnt)
-{
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsets; s += gridDim.x * blockDim.x)
-        cnt[s * CNT_N + CNT_STATUS] = *sets[s].status;
-}
-
 // Survivors of the energy cull (flags over the batch's contours), their count
-// and largest radius per set (float bits of R > 0 order like ints; one atomic
-// per warp).  Block row blockIdx.y is set blockIdx.y; launched with whole warps.
-__global__ void flag_kernel(const LocSet *sets, uint8_t *flags, int32_t *cnt)
+// and largest radius per set (float bits of R > 0 order like ints), and the set's
+// status word.  Block row blockIdx.y is set blockIdx.y.  Reads 8 bytes a contour; one
+// pair of atomics per block, since one per warp serialised on the set's two counters
+// (1.4 M contours: 46 us).
+__global__ void __launch_bounds__(256) flag_kernel(const LocSet *sets, uint8_t *flags, int32_t *cnt)
 {
     const LocSet &S = sets[blockIdx.y];
     const float *E = S.state + 4 * S.C, *R = S.state + 3 * S.C;
+    int32_t *c = cnt + (int64_t)blockIdx.y * CNT_N;
+    if (blockIdx.x == 0 && threadIdx.x == 0) c[CNT_STATUS] = *S.status;
     int32_t nk = 0, mx = 0;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < S.C; k += (int64_t)gridDim.x * blockDim.x) {
         const float e = E[k];
@@ -105,11 +105,21 @@ __global__ void flag_kernel(const LocSet *sets, uint8_t *flags, int32_t *cnt)
             mx = max(mx, __float_as_int(R[k]));
         }
     }
+    __shared__ int32_t wn[8], wm[8];
     nk = __reduce_add_sync(0xffffffffu, nk);
     mx = __reduce_max_sync(0xffffffffu, mx);
     if ((threadIdx.x & 31) == 0) {
-        if (nk) atomicAdd(&cnt[blockIdx.y * CNT_N + CNT_SURV], nk);
-        if (mx > 0) atomicMax(&cnt[blockIdx.y * CNT_N + CNT_MAXR], mx);
+        wn[threadIdx.x >> 5] = nk;
+        wm[threadIdx.x >> 5] = mx;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) {
+            nk += wn[w];
+            mx = max(mx, wm[w]);
+        }
+        if (nk) atomicAdd(&c[CNT_SURV], nk);
+        if (mx > 0) atomicMax(&c[CNT_MAXR], mx);
     }
 }
 
@@ -128,102 +138,156 @@ __global__ void key_kernel(const LocSet *sets, int nsets, const int32_t *surv, i
     }
 }
 
-// positions in priority order
-__global__ void positions_kernel(const LocSet *sets, int nsets, const int32_t *order, int64_t n, float4 *pos)
-{
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        const LocSet &S = sets[set_of<&LocSet::sbase>(sets, nsets, p)];
-        const int64_t k = order[p] - S.cbase;
-        pos[p] = make_float4(S.state[k], S.state[S.C + k], S.state[2 * S.C + k], S.state[3 * S.C + k]);
-    }
-}
-
 __device__ __forceinline__ int cell_axis(float x, float inv_h, int nc)
 {
     int i = (int)floorf(x * inv_h);
     return i < 0 ? 0 : (i >= nc ? nc - 1 : i);
 }
 
-__global__ void cell_kernel(const LocSet *sets, int nsets, const float4 *pos, int64_t n, uint32_t *cellk,
-                            uint32_t *celli)
+// Positions in priority order, each survivor's grid cell and its rank in the cell
+// (`count` per cell, cleared before)
+__global__ void cell_count_kernel(const LocSet *sets, int nsets, const int32_t *order, int64_t n, float4 *pos,
+                                  uint32_t *cell, uint32_t *rank, int32_t *count)
 {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
         const LocSet &S = sets[set_of<&LocSet::sbase>(sets, nsets, p)];
-        const float4 q = pos[p];
+        const int64_t k = order[p] - S.cbase;
+        const float4 q = make_float4(S.state[k], S.state[S.C + k], S.state[2 * S.C + k], S.state[3 * S.C + k]);
+        pos[p] = q;
         const int cx = cell_axis(q.x, S.g.inv_h, S.g.nc[0]);
         const int cy = cell_axis(q.y, S.g.inv_h, S.g.nc[1]);
         const int cz = cell_axis(q.z, S.g.inv_h, S.g.nc[2]);
-        cellk[p] = (uint32_t)(S.cellbase + cx + (int64_t)S.g.nc[0] * (cy + (int64_t)S.g.nc[1] * cz));
-        celli[p] = (uint32_t)p;
+        const int64_t c = S.cellbase + cx + (int64_t)S.g.nc[0] * (cy + (int64_t)S.g.nc[1] * cz);
+        cell[p] = (uint32_t)c;
+        rank[p] = (uint32_t)atomicAdd(&count[c], 1);
     }
 }
 
-__global__ void cell_start_kernel(const uint32_t *cellk_sorted, int64_t n, int64_t ncells, int32_t *start)
+// The survivors and their positions by cell (in any order within a cell)
+__global__ void cell_scatter_kernel(int64_t n, const uint32_t *cell, const uint32_t *rank, const int32_t *start,
+                                    const float4 *pos, uint32_t *list, float4 *list_pos)
 {
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c <= ncells; c += (int64_t)gridDim.x * blockDim.x) {
-        int64_t lo = 0, hi = n;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            if ((int64_t)cellk_sorted[mid] < c) lo = mid + 1; else hi = mid;
-        }
-        start[c] = (int32_t)lo;
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = (int64_t)start[cell[p]] + rank[p];
+        list[j] = (uint32_t)p;
+        list_pos[j] = pos[p];
     }
 }
 
 // One round of the parallel greedy competition over the survivors of every set.
 // A set's cells hold only its own survivors, and within a set batch order is
-// priority order.  `undecided` counts per set what is still open.
-__global__ void round_kernel(const LocSet *sets, int nsets, const float4 *pos, int64_t n, const int32_t *start,
-                             const uint32_t *celli_sorted, uint8_t *status, int32_t *undecided)
+// priority order.  CNT_OPEN counts per set what is still open.
+//
+// A warp per survivor.  The three cells of a row along x are neighbours in the list, so
+// a survivor's 27 cells are 9 ranges: lanes 0-8 read their bounds, and the lanes then
+// share the entries.  Bound by the latency of the chain bounds -> entry -> status: one
+// thread per survivor walked 27 cells of it one after the other, and every link of a
+// chain of competing contours cost a launch.  Here a warp that waits for a neighbour
+// looks again up to LOOKS times, re-reading only the neighbours still open (two per
+// lane are kept; with more it reads everything again); what is open after that is left
+// to the next round, so nothing depends on which blocks run together.  2,048 contours
+// (about 770 survivors): the rounds of a call 168 -> 15 us; 1.4 M (540 thousand
+// survivors): 557 -> 240 us.
+constexpr int LOOKS = 64;
+constexpr uint32_t NONE = 0xffffffffu;
+
+__global__ void __launch_bounds__(256) round_kernel(const LocSet *sets, int nsets, const float4 *pos, int64_t n,
+                                                    const int32_t *start, const uint32_t *list, const float4 *list_pos,
+                                                    uint8_t *status, int32_t *cnt)
 {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        if (status[p] != UNDECIDED) continue;
-        const int s = set_of<&LocSet::sbase>(sets, nsets, p);
-        const LocSet &S = sets[s];
-        const Grid &g = S.g;
-        const float4 a = pos[p];
-        const int cx = cell_axis(a.x, g.inv_h, g.nc[0]);
-        const int cy = cell_axis(a.y, g.inv_h, g.nc[1]);
-        const int cz = cell_axis(a.z, g.inv_h, g.nc[2]);
-        bool rejected = false, pending = false;
-        for (int dz = -1; dz <= 1 && !rejected; ++dz) {
-            const int z = cz + dz;
-            if (z < 0 || z >= g.nc[2]) continue;
-            for (int dy = -1; dy <= 1 && !rejected; ++dy) {
-                const int y = cy + dy;
-                if (y < 0 || y >= g.nc[1]) continue;
-                for (int dx = -1; dx <= 1 && !rejected; ++dx) {
-                    const int x = cx + dx;
-                    if (x < 0 || x >= g.nc[0]) continue;
-                    const int64_t c = S.cellbase + x + (int64_t)g.nc[0] * (y + (int64_t)g.nc[1] * z);
-                    for (int32_t j = start[c]; j < start[c + 1]; ++j) {
-                        const uint32_t q = celli_sorted[j];
-                        if ((int64_t)q >= p) continue;   // only higher priority
-                        const float4 b = pos[q];
-                        const float ex = a.x - b.x, ey = a.y - b.y, ez = a.z - b.z;
-                        const float dist = sqrtf(ex * ex + ey * ey + ez * ez);
-                        if (!(dist < S.rho * fmaxf(a.w, b.w))) continue;
-                        const uint8_t sq = *(volatile const uint8_t *)&status[q];
-                        if (sq == ACCEPTED) {
-                            rejected = true;
-                            break;
+    const int64_t p = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (p >= n || status[p] != UNDECIDED) return;   // the same for the whole warp
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int s = set_of<&LocSet::sbase>(sets, nsets, p);
+    const LocSet &S = sets[s];
+    const Grid &g = S.g;
+    const float rho = S.rho;
+    const float4 a = pos[p];
+    int from = 0, len = 0;   // lanes 0-8: a row of up to three cells
+    if (lane < 9) {
+        const int x = cell_axis(a.x, g.inv_h, g.nc[0]);
+        const int y = cell_axis(a.y, g.inv_h, g.nc[1]) + lane % 3 - 1;
+        const int z = cell_axis(a.z, g.inv_h, g.nc[2]) + lane / 3 - 1;
+        if (y >= 0 && y < g.nc[1] && z >= 0 && z < g.nc[2]) {
+            const int64_t row = S.cellbase + (int64_t)g.nc[0] * (y + (int64_t)g.nc[1] * z);
+            from = start[row + max(x - 1, 0)];
+            len = start[row + min(x + 1, g.nc[0] - 1) + 1] - from;
+        }
+    }
+    int upto = len;   // entries up to and including this lane's row
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+        const int v = __shfl_up_sync(all, upto, o);
+        if (lane >= o) upto += v;
+    }
+    const int total = __shfl_sync(all, upto, 8);
+    const int shift = from - (upto - len);   // entry number to list index
+    volatile const uint8_t *st = status;
+    bool rejected = false, full = false;   // full: more open neighbours than the lane keeps
+    uint32_t q0 = NONE, q1 = NONE;
+    auto scan = [&]() {
+        q0 = q1 = NONE;
+        full = false;
+        for (int base = 0; base < total; base += 32) {
+            const int e = base + lane;
+            int row = 0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) row += e >= __shfl_sync(all, upto, i) ? 1 : 0;
+            const int j = e + __shfl_sync(all, shift, row);
+            if (e < total) {
+                const uint32_t q = list[j];
+                const float4 b = list_pos[j];   // with q, not after it
+                if ((int64_t)q < p) {           // only higher priority
+                    const float ex = a.x - b.x, ey = a.y - b.y, ez = a.z - b.z;
+                    const float dist = sqrtf(ex * ex + ey * ey + ez * ez);
+                    if (dist < rho * fmaxf(a.w, b.w)) {
+                        const uint8_t sq = st[q];
+                        if (sq == ACCEPTED) rejected = true;
+                        if (sq == UNDECIDED) {
+                            if (q0 == NONE) q0 = q;
+                            else if (q1 == NONE) q1 = q;
+                            else full = true;
                         }
-                        if (sq == UNDECIDED) pending = true;
                     }
                 }
             }
+            if (__any_sync(all, rejected)) return;
         }
-        if (rejected) status[p] = REJECTED;
-        else if (!pending) status[p] = ACCEPTED;
-        else atomicAdd(&undecided[s], 1);
+    };
+    scan();
+    for (int look = 0; look < LOOKS; ++look) {
+        if (__any_sync(all, rejected)) {
+            if (lane == 0) *(volatile uint8_t *)&status[p] = REJECTED;
+            return;
+        }
+        if (!__any_sync(all, q0 != NONE || q1 != NONE)) {
+            if (lane == 0) *(volatile uint8_t *)&status[p] = ACCEPTED;
+            return;
+        }
+        __nanosleep(100);
+        if (__any_sync(all, full)) {
+            scan();
+            continue;
+        }
+        if (q0 != NONE) {
+            const uint8_t sq = st[q0];
+            if (sq == ACCEPTED) rejected = true;
+            if (sq != UNDECIDED) q0 = NONE;
+        }
+        if (q1 != NONE) {
+            const uint8_t sq = st[q1];
+            if (sq == ACCEPTED) rejected = true;
+            if (sq != UNDECIDED) q1 = NONE;
+        }
     }
+    if (lane == 0) atomicAdd(&cnt[(int64_t)s * CNT_N + CNT_OPEN], 1);
 }
 
-__global__ void accepted_flags_kernel(const uint8_t *status, int64_t n, uint8_t *flags)
-{
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
-        flags[p] = status[p] == ACCEPTED ? 1 : 0;
-}
+struct IsAccepted {
+    const uint8_t *status;
+    __device__ __forceinline__ bool operator()(int32_t p) const { return status[p] == ACCEPTED; }
+};
 
 __device__ __forceinline__ int64_t lower_bound_i32(const int32_t *a, int64_t n, int64_t key)
 {
@@ -241,8 +305,8 @@ __global__ void accepted_ranges_kernel(const LocSet *sets, int nsets, const int3
                                        int32_t *cnt)
 {
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsets; s += gridDim.x * blockDim.x) {
-        const int64_t b = lower_bound_i32(acc, *m, sets[s].sbase);
-        const int64_t e = lower_bound_i32(acc, *m, sets[s].sbase + sets[s].n);
+        const int64_t b = s == 0 ? 0 : lower_bound_i32(acc, *m, sets[s].sbase);
+        const int64_t e = s == nsets - 1 ? *m : lower_bound_i32(acc, *m, sets[s].sbase + sets[s].n);
         cnt[s * CNT_N + CNT_ABASE] = (int32_t)b;
         cnt[s * CNT_N + CNT_ACC] = (int32_t)(e - b);
     }
@@ -310,7 +374,6 @@ ac_status localize_many(ac_contours *const *sets, const float *E0, ac_cell *cons
     LC_CUDA(sc.hsets.ensure(sizeof(LocSet) * nsets));
     LC_CUDA(sc.counters.ensure(sizeof(int32_t) * cnt_ints));
     LC_CUDA(sc.hcount.ensure(sizeof(int32_t) * cnt_ints));
-    LC_CUDA(sc.und.ensure(sizeof(int32_t) * nsets));
     LocSet *dsets = sc.lsets.as<LocSet>();
     int32_t *cnt = sc.counters.as<int32_t>();
     int32_t *h = sc.hcount.as<int32_t>();
@@ -321,16 +384,13 @@ ac_status localize_many(ac_contours *const *sets, const float *E0, ac_cell *cons
     std::memcpy(sc.hsets.p, L.data(), sizeof(LocSet) * nsets);
     LC_CUDA(cudaMemcpyAsync(dsets, sc.hsets.p, sizeof(LocSet) * nsets, cudaMemcpyHostToDevice, st));
     LC_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * cnt_ints, st));
-    status_kernel<<<blocks_for(nsets), 256, 0, st>>>(dsets, nsets, cnt);
+    LC_CUDA(sc.flags.ensure(total));
+    const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>((maxC + 255) / 256, 1216));
+    flag_kernel<<<dim3(bx, (unsigned)nsets), 256, 0, st>>>(dsets, sc.flags.as<uint8_t>(), cnt);
     count_launch();
     LC_CUDA(cudaGetLastError());
     if (total > 0) {
-        LC_CUDA(sc.flags.ensure(total));
         LC_CUDA(sc.surv.ensure(sizeof(int32_t) * total));
-        const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>((maxC + 255) / 256, 4096));
-        flag_kernel<<<dim3(bx, (unsigned)nsets), 256, 0, st>>>(dsets, sc.flags.as<uint8_t>(), cnt);
-        count_launch();
-        LC_CUDA(cudaGetLastError());
         thrust::counting_iterator<int32_t> iota(0);
         size_t tmp = 0;
         LC_CUDA(cub::DeviceSelect::Flagged(nullptr, tmp, iota, sc.flags.as<uint8_t>(), sc.surv.as<int32_t>(), tot,
@@ -396,92 +456,81 @@ ac_status localize_many(ac_contours *const *sets, const float *E0, ac_cell *cons
     LC_CUDA(cub::DeviceRadixSort::SortPairs(sc.cub.p, tmp, ek, ek + n, sc.surv.as<int32_t>(), order, (int)n, 0,
                                             key_bits, st));
     LC_CUDA(sc.pos.ensure(sizeof(float4) * n));
-    float4 *pos = sc.pos.as<float4>();
-    positions_kernel<<<blocks_for(n), 256, 0, st>>>(dsets, nsets, order, n, pos);
-    count_launch();
-    LC_CUDA(cudaGetLastError());
+    LC_CUDA(sc.list_pos.ensure(sizeof(float4) * n));
     LC_CUDA(sc.cellk.ensure(sizeof(uint32_t) * n));
-    LC_CUDA(sc.cellk_s.ensure(sizeof(uint32_t) * n));
     LC_CUDA(sc.celli.ensure(sizeof(uint32_t) * n));
-    LC_CUDA(sc.celli_s.ensure(sizeof(uint32_t) * n));
+    LC_CUDA(sc.list.ensure(sizeof(uint32_t) * n));
     LC_CUDA(sc.cell_start.ensure(sizeof(int32_t) * (ncells + 1)));
-    cell_kernel<<<blocks_for(n), 256, 0, st>>>(dsets, nsets, pos, n, sc.cellk.as<uint32_t>(), sc.celli.as<uint32_t>());
+    float4 *pos = sc.pos.as<float4>();
+    int32_t *start = sc.cell_start.as<int32_t>();
+    LC_CUDA(cudaMemsetAsync(start, 0, sizeof(int32_t) * (ncells + 1), st));
+    cell_count_kernel<<<blocks_for(n), 256, 0, st>>>(dsets, nsets, order, n, pos, sc.cellk.as<uint32_t>(),
+                                                     sc.celli.as<uint32_t>(), start);
     count_launch();
     LC_CUDA(cudaGetLastError());
-    const int cell_bits = bits_for((uint64_t)ncells);
     tmp = 0;
-    LC_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tmp, sc.cellk.as<uint32_t>(), sc.cellk_s.as<uint32_t>(),
-                                            sc.celli.as<uint32_t>(), sc.celli_s.as<uint32_t>(), (int)n, 0, cell_bits,
-                                            st));
+    LC_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tmp, start, start, (int)(ncells + 1), st));
     LC_CUDA(sc.cub.ensure(tmp));
-    LC_CUDA(cub::DeviceRadixSort::SortPairs(sc.cub.p, tmp, sc.cellk.as<uint32_t>(), sc.cellk_s.as<uint32_t>(),
-                                            sc.celli.as<uint32_t>(), sc.celli_s.as<uint32_t>(), (int)n, 0, cell_bits,
-                                            st));
-    cell_start_kernel<<<blocks_for(ncells + 1), 256, 0, st>>>(sc.cellk_s.as<uint32_t>(), n, ncells,
-                                                              sc.cell_start.as<int32_t>());
+    LC_CUDA(cub::DeviceScan::ExclusiveSum(sc.cub.p, tmp, start, start, (int)(ncells + 1), st));
+    cell_scatter_kernel<<<blocks_for(n), 256, 0, st>>>(n, sc.cellk.as<uint32_t>(), sc.celli.as<uint32_t>(), start, pos,
+                                                       sc.list.as<uint32_t>(), sc.list_pos.as<float4>());
     count_launch();
     LC_CUDA(cudaGetLastError());
 
     // 4. rounds until every survivor is decided.  Each round decides at least the
     //    undecided survivor of highest priority of every set, so the largest set's
     //    n rounds settle all; the bound (that n + 8 unless a test lowers it) is
-    //    checked between batches of up to eight rounds.
+    //    checked between rounds.  After each round the kept survivors are collected in
+    //    batch (= per set, acceptance) order, with each set's range of them, on the
+    //    assumption that it was the last; few cells are copied back with the counts.
     LC_CUDA(sc.stat.ensure(n));
+    LC_CUDA(sc.acc.ensure(sizeof(int32_t) * n));
+    LC_CUDA(sc.cells.ensure(sizeof(ac_cell) * n));
+    LC_CUDA(sc.hcells.ensure(sizeof(ac_cell) * n));
     uint8_t *status = sc.stat.as<uint8_t>();
-    int32_t *und = sc.und.as<int32_t>();
-    int32_t *hund = h;   // the page-locked counts are read: reused for the undecided counts
+    int32_t *acc = sc.acc.as<int32_t>();
+    thrust::counting_iterator<int32_t> iota(0);
+    const IsAccepted accepted{status};
+    tmp = 0;
+    LC_CUDA(cub::DeviceSelect::If(nullptr, tmp, iota, acc, tot + 1, (int)n, accepted, st));
+    LC_CUDA(sc.cub.ensure(tmp));
     LC_CUDA(cudaMemsetAsync(status, UNDECIDED, n, st));
     const int64_t max_rounds = localize_round_limit(n_max);
+    const bool few = n <= 16384;   // 400 KB of cells: less than another synchronisation costs
     int64_t rounds = 0;
-    for (bool open = true; open;) {
+    for (bool open = true; open; ++rounds) {
         if (rounds >= max_rounds) {
             const int32_t bit = STATUS_LOCALIZE_LIMIT;
             for (int s = 0; s < nsets; ++s)
-                if (L[(size_t)s].n > 0 && (rounds == 0 || hund[s] > 0))
+                if (L[(size_t)s].n > 0 && (rounds == 0 || h[s * CNT_N + CNT_OPEN] > 0))
                     LC_CUDA(cudaMemcpyAsync(sets[s]->status, &bit, sizeof(bit), cudaMemcpyHostToDevice, st));
             LC_CUDA(cudaStreamSynchronize(st));
             LC_FAIL(AC_ERR_TIMEOUT, "ac_localize: competition did not settle within its round bound");
         }
-        const int64_t batch = std::min<int64_t>(8, max_rounds - rounds);
-        for (int64_t r = 0; r < batch; ++r, ++rounds) {
-            LC_CUDA(cudaMemsetAsync(und, 0, sizeof(int32_t) * nsets, st));
-            round_kernel<<<blocks_for(n), 256, 0, st>>>(dsets, nsets, pos, n, sc.cell_start.as<int32_t>(),
-                                                        sc.celli_s.as<uint32_t>(), status, und);
-            count_launch();
-            LC_CUDA(cudaGetLastError());
-        }
-        LC_CUDA(cudaMemcpyAsync(hund, und, sizeof(int32_t) * nsets, cudaMemcpyDeviceToHost, st));
+        if (rounds > 0)
+            LC_CUDA(cudaMemset2DAsync(cnt + CNT_OPEN, sizeof(int32_t) * CNT_N, 0, sizeof(int32_t), nsets, st));
+        round_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(dsets, nsets, pos, n, start, sc.list.as<uint32_t>(),
+                                                              sc.list_pos.as<float4>(), status, cnt);
+        count_launch();
+        LC_CUDA(cudaGetLastError());
+        LC_CUDA(cub::DeviceSelect::If(sc.cub.p, tmp, iota, acc, tot + 1, (int)n, accepted, st));
+        accepted_ranges_kernel<<<blocks_for(nsets), 256, 0, st>>>(dsets, nsets, acc, tot + 1, cnt);
+        count_launch();
+        LC_CUDA(cudaGetLastError());
+        cells_kernel<<<blocks_for(n), 256, 0, st>>>(dsets, nsets, pos, order, acc, tot + 1, sc.cells.as<ac_cell>());
+        count_launch();
+        LC_CUDA(cudaGetLastError());
+        LC_CUDA(cudaMemcpyAsync(h, cnt, sizeof(int32_t) * cnt_ints, cudaMemcpyDeviceToHost, st));
+        if (few)
+            LC_CUDA(cudaMemcpyAsync(sc.hcells.p, sc.cells.p, sizeof(ac_cell) * n, cudaMemcpyDeviceToHost, st));
         LC_CUDA(cudaStreamSynchronize(st));
         open = false;
-        for (int s = 0; s < nsets; ++s) open = open || hund[s] > 0;
+        for (int s = 0; s < nsets; ++s) open = open || h[s * CNT_N + CNT_OPEN] > 0;
     }
 
-    // 5. the kept survivors in batch (= per set, acceptance) order, each set's
-    //    range of them, and the cells, copied back after the counts
-    LC_CUDA(sc.acc.ensure(sizeof(int32_t) * n));
-    accepted_flags_kernel<<<blocks_for(n), 256, 0, st>>>(status, n, sc.flags.as<uint8_t>());
-    count_launch();
-    LC_CUDA(cudaGetLastError());
-    thrust::counting_iterator<int32_t> iota(0);
-    tmp = 0;
-    LC_CUDA(cub::DeviceSelect::Flagged(nullptr, tmp, iota, sc.flags.as<uint8_t>(), sc.acc.as<int32_t>(), tot + 1,
-                                       (int)n, st));
-    LC_CUDA(sc.cub.ensure(tmp));
-    LC_CUDA(cub::DeviceSelect::Flagged(sc.cub.p, tmp, iota, sc.flags.as<uint8_t>(), sc.acc.as<int32_t>(), tot + 1,
-                                       (int)n, st));
-    accepted_ranges_kernel<<<blocks_for(nsets), 256, 0, st>>>(dsets, nsets, sc.acc.as<int32_t>(), tot + 1, cnt);
-    count_launch();
-    LC_CUDA(cudaGetLastError());
-    LC_CUDA(sc.cells.ensure(sizeof(ac_cell) * n));
-    LC_CUDA(sc.hcells.ensure(sizeof(ac_cell) * n));
-    cells_kernel<<<blocks_for(n), 256, 0, st>>>(dsets, nsets, pos, order, sc.acc.as<int32_t>(), tot + 1,
-                                                sc.cells.as<ac_cell>());
-    count_launch();
-    LC_CUDA(cudaGetLastError());
-    LC_CUDA(cudaMemcpyAsync(h, cnt, sizeof(int32_t) * cnt_ints, cudaMemcpyDeviceToHost, st));
-    LC_CUDA(cudaStreamSynchronize(st));
-    const int64_t M = h[(size_t)nsets * CNT_N + 1];   // the cells, contiguous, set by set
-    if (M > 0) {
+    // 5. the cells, contiguous, set by set
+    const int64_t M = h[(size_t)nsets * CNT_N + 1];
+    if (M > 0 && !few) {
         LC_CUDA(cudaMemcpyAsync(sc.hcells.p, sc.cells.p, sizeof(ac_cell) * M, cudaMemcpyDeviceToHost, st));
         LC_CUDA(cudaStreamSynchronize(st));
     }
