@@ -9,6 +9,14 @@
 // (y, z), skips rows that miss the ball, and its lanes take consecutive voxels of
 // a row's chord, so a row is read with neighbouring addresses.  Gathers go
 // through the read-only cache from global memory.
+//
+// Bound by instruction issue (72-76 % of the slots before and after): a voxel cost 55
+// instructions, of which the square root and the division, with their paths for special
+// operands, were 22 and most of the branches; in 3D a row whose chord ends between a
+// lane's two voxels ran once for the lanes with both and once for the others.  Now the
+// two voxels of a step share packed instructions, the reciprocal root serves both root
+// and quotient, and a lane without a second voxel adds its first in the same
+// instructions.  10 iterations: 1024^2 u8 263 -> 143 us, 256x250x64 u16 1720 -> 1042 us.
 #include "ac_evolve.cuh"
 #include "ac_host.h"
 
@@ -20,7 +28,7 @@ __device__ __forceinline__ Step eval_grid(const VolDesc &V, const EvolveArgs &a,
                                           unsigned mask)
 {
     const float Ro = R + 0.5f * a.dR;
-    const float Ro2 = Ro * Ro;
+    const float Ro2 = __fmul_rn(Ro, Ro);
     int lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
@@ -37,55 +45,62 @@ __device__ __forceinline__ Step eval_grid(const VolDesc &V, const EvolveArgs &a,
         const int zz = DIM == 3 ? min(max(kz, 0), V.n[2] - 1) : 0;
         for (int jy = lo[1]; jy <= hi[1]; ++jy) {
             const float dy = fmaf((float)jy, V.sp[1], -c[1]);
-            const float rem = Ro2 - fmaf(dy, dy, dz * dz);
+            const float q = __fmaf_rn(dy, dy, __fmul_rn(dz, dz));
+            const float rem = __fsub_rn(Ro2, q);   // not fused: decides which voxels a chord ends on
             if (rem < 0.0f) continue;   // the row misses the ball (same for the whole group)
-            const float chord = sqrtf(rem);
+            const float chord = sqrt1(fmaxf(rem, ROOT_MIN));
             const int i0 = (int)ceilf((c[0] - chord) * V.inv_sp[0]);
             const int i1 = (int)floorf((c[0] + chord) * V.inv_sp[0]);
             const int yy = min(max(jy, 0), V.n[1] - 1);
             const int64_t row = (int64_t)zz * V.pitch_z + (int64_t)yy * V.pitch_y;
-            // the terms of voxel ix of this row
-            auto terms = [&](int ix, float *v) {
-                const float dx = fmaf((float)ix, V.sp[0], -c[0]);
-                const float I = ix <= i1 ? ldg_f<T>(data + checked(row + min(max(ix, 0), V.n[0] - 1), nvox, V.status))
-                                         : 0.0f;
-                const float r = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-                const float t1 = fmaf(r, a.inv_dr, B1), t2 = fmaf(r, a.inv_dR, B2);
-                const float r1 = __saturatef(t1), r2 = __saturatef(t2);
-                const float S = fmaf(2.0f, r1, -1.0f) - r2;
-                const bool b1 = r1 == t1, b2 = r2 == t2;   // voxel inside the inner / outer band
-                const float dSdR = (b1 ? a.kR1 : 0.0f) + (b2 ? a.kR2 : 0.0f);
-                // -S'(r) I / r: the direction (x - c) / r without a division by zero at the centre
-                const float g = r > 0.0f ? ((b1 ? a.kr1 : 0.0f) + (b2 ? a.kr2 : 0.0f)) * I / r : 0.0f;
-                v[0] = S * I;
-                v[1] = dSdR * I;
-                v[2] = g * dx;
-                v[3] = g * dy;
-                v[4] = g * dz;
-            };
-            // two voxels per step (ix and ix + G), summed in one rounding before the
-            // compensated addition: two independent chains of work per lane.  In 2D
-            // every step takes a pair (a voxel beyond the chord adds zero: cheaper than
-            // a divergent tail on these latency-bound rows); in 3D, whose rows are
-            // shorter, pairs only while both voxels lie on the chord, then a single one
-            int ix = i0 + lig;
-            for (; DIM == 2 ? ix <= i1 : ix + G <= i1; ix += 2 * G) {
-                float v[5], w[5];
-                terms(ix, v);
-                terms(ix + G, w);
+            // Two voxels of the row per step (ix and ix + G), side by side in packed
+            // instructions: two independent chains of work per lane, and the products are
+            // summed in one rounding before the compensated addition.  In 2D a second voxel
+            // beyond the chord adds zero; in 3D, whose rows are shorter, the first is then
+            // added alone, in the same instructions.
+            for (int ix = i0 + lig; ix <= i1; ix += 2 * G) {
+                const bool two = ix + G <= i1;
+                const float fx = (float)ix;
+                const float2 dx = fma2(make_float2(fx, fx + (float)G), dup2(V.sp[0]), dup2(-c[0]));
+                const float Iv = ldg_f<T>(data + checked(row + min(max(ix, 0), V.n[0] - 1), nvox, V.status));
+                const float Iw = two ? ldg_f<T>(data + checked(row + min(max(ix + G, 0), V.n[0] - 1), nvox, V.status))
+                                     : 0.0f;
+                const float2 d2 = fma2(dx, dx, dup2(q));
+                float2 rs;
+                const float2 r = sqrt2(make_float2(fmaxf(d2.x, ROOT_MIN), fmaxf(d2.y, ROOT_MIN)), rs);
+                const float2 t1 = fma2(r, dup2(a.inv_dr), dup2(B1)), t2 = fma2(r, dup2(a.inv_dR), dup2(B2));
+                const float2 s1 = make_float2(__saturatef(t1.x), __saturatef(t1.y));
+                const float2 s2 = make_float2(__saturatef(t2.x), __saturatef(t2.y));
+                const float2 S = sub2(fma2(dup2(2.0f), s1, dup2(-1.0f)), s2);
+                // voxel inside the inner / outer band
+                const bool v1 = s1.x == t1.x, v2 = s2.x == t2.x, w1 = s1.y == t1.y, w2 = s2.y == t2.y;
+                const float2 dSdR = add2(make_float2(v1 ? a.kR1 : 0.0f, w1 ? a.kR1 : 0.0f),
+                                         make_float2(v2 ? a.kR2 : 0.0f, w2 ? a.kR2 : 0.0f));
+                // -S'(r) I / r, for the direction (x - c) / r (zero for a voxel on the centre)
+                const float2 k = add2(make_float2(v1 ? a.kr1 : 0.0f, w1 ? a.kr1 : 0.0f),
+                                      make_float2(v2 ? a.kr2 : 0.0f, w2 ? a.kr2 : 0.0f));
+                const float2 g = div2(make_float2(__fmul_rn(d2.x > ROOT_MIN ? k.x : 0.0f, Iv),
+                                                  __fmul_rn(d2.y > ROOT_MIN ? k.y : 0.0f, Iw)), r, rs);
+                const float gv = g.x, gw = g.y;
+                const float fv[5] = {S.x, dSdR.x, gv, gv, gv}, xv[5] = {Iv, Iv, dx.x, dy, dz};
+                const float fw[5] = {S.y, dSdR.y, gw, gw, gw}, xw[5] = {Iw, Iw, dx.y, dy, dz};
+                // which voxel's product is fused with the sum of the two
+                constexpr bool w_first[5] = {true, false, true, false, false};
 #pragma unroll
                 for (int m = 0; m < (DIM == 3 ? 5 : 4); ++m) {
-                    if (COMP) kadd(acc[m], v[m] + w[m]);
-                    else acc[m].s += v[m] + w[m];
-                }
-            }
-            if (ix <= i1) {
-                float v[5];
-                terms(ix, v);
-#pragma unroll
-                for (int m = 0; m < (DIM == 3 ? 5 : 4); ++m) {
-                    if (COMP) kadd(acc[m], v[m]);
-                    else acc[m].s += v[m];
+                    const bool alone = DIM == 3 && !two;
+                    const float w = w_first[m] ? __fmul_rn(fv[m], xv[m]) : __fmul_rn(fw[m], xw[m]);
+                    const float ff = w_first[m] && !alone ? fw[m] : fv[m], fi = w_first[m] && !alone ? xw[m] : xv[m];
+                    if (COMP) {
+                        float y = __fmaf_rn(ff, fi, alone ? -acc[m].c : w);
+                        if (!alone) y = y - acc[m].c;
+                        const float t = acc[m].s + y;
+                        acc[m].c = (t - acc[m].s) - y;
+                        acc[m].s = t;
+                    } else {
+                        const float y = __fmaf_rn(ff, fi, alone ? acc[m].s : w);
+                        acc[m].s = alone ? y : acc[m].s + y;
+                    }
                 }
             }
         }
