@@ -47,33 +47,6 @@ __device__ __forceinline__ void clear_counts(unsigned long long *c)
     if (blockIdx.x == 0 && threadIdx.x < 3) c[threadIdx.x] = 0;
 }
 
-// Exclusive prefix sum of one value per thread over the block (blockDim.x a multiple
-// of 32, at most 1024); *total is the sum over the block.
-__device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t *warp_sums, uint32_t *total)
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_sums[w] = x;
-    __syncthreads();
-    if (w == 0) {
-        uint32_t s = lane < nw ? warp_sums[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        warp_sums[lane] = s;   // inclusive; warp_sums holds 32 values
-    }
-    __syncthreads();
-    *total = warp_sums[31];
-    return x - v + (w ? warp_sums[w - 1] : 0);
-}
-
 // Few contours and bricks: one CTA counts in shared memory, scans and scatters, each
 // thread keeping its contours' (brick, rank) in registers: one launch instead of a clear
 // and three.  12 contours a thread is what its 64 registers hold without spills to speak of.
