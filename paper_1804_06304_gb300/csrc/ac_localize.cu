@@ -217,14 +217,17 @@ __global__ void cell_count_kernel(const LocSet *sets, int nsets, const int32_t *
     }
 }
 
-// The survivors and their positions by cell (in any order within a cell)
-__global__ void cell_scatter_kernel(int64_t n, const uint32_t *cell, const uint32_t *rank, const int32_t *start,
-                                    const float4 *pos, uint32_t *list, float4 *list_pos)
+// The survivors, their positions and their states by cell (in any order within a cell);
+// `rank` becomes a survivor's place in the list
+__global__ void cell_scatter_kernel(int64_t n, const uint32_t *cell, uint32_t *rank, const int32_t *start,
+                                    const float4 *pos, uint32_t *list, float4 *list_pos, uint8_t *list_status)
 {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = (int64_t)start[cell[p]] + rank[p];
         list[j] = (uint32_t)p;
         list_pos[j] = pos[p];
+        list_status[j] = UNDECIDED;
+        rank[p] = (uint32_t)j;
     }
 }
 
@@ -234,30 +237,34 @@ __global__ void cell_scatter_kernel(int64_t n, const uint32_t *cell, const uint3
 //
 // A warp per survivor.  The three cells of a row along x are neighbours in the list, so
 // a survivor's 27 cells are 9 ranges: lanes 0-8 read their bounds, and the lanes then
-// share the entries.  Bound by the latency of the chain bounds -> entry -> status: one
+// share the entries.  Bound by the latency of the chain position -> bounds -> entry (the
+// states lie by list place too, so that they come with the entry and not after it): one
 // thread per survivor walked 27 cells of it one after the other, and every link of a
 // chain of competing contours cost a launch.  Here a warp that waits for a neighbour
 // looks again up to LOOKS times, re-reading only the neighbours still open (two per
 // lane are kept; with more it reads everything again); what is open after that is left
 // to the next round, so nothing depends on which blocks run together.  2,048 contours
-// (about 770 survivors): the rounds of a call 168 -> 15 us; 1.4 M (540 thousand
-// survivors): 557 -> 240 us.
+// (about 770 survivors): the rounds of a call 168 -> 11 us; 1.4 M (540 thousand
+// survivors): 557 -> 165 us (240 us with the states by priority alone).
 constexpr int LOOKS = 64;
 constexpr uint32_t NONE = 0xffffffffu;
 
 __global__ void __launch_bounds__(256) round_kernel(const LocSet *sets, int nsets, const float4 *pos, int64_t n,
                                                     const int32_t *start, const uint32_t *list, const float4 *list_pos,
-                                                    uint8_t *status, int32_t *cnt)
+                                                    const uint32_t *place, uint8_t *list_status, uint8_t *status,
+                                                    int32_t *cnt)
 {
     const int64_t p = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (p >= n || status[p] != UNDECIDED) return;   // the same for the whole warp
+    if (p >= n) return;
+    const float4 a = pos[p];
+    const uint32_t mine = place[p];
+    if (status[p] != UNDECIDED) return;   // the same for the whole warp
     const unsigned all = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int s = set_of<&LocSet::sbase>(sets, nsets, p);
     const LocSet &S = sets[s];
     const Grid &g = S.g;
     const float rho = S.rho;
-    const float4 a = pos[p];
     int from = 0, len = 0;   // lanes 0-8: a row of up to three cells
     if (lane < 9) {
         const int x = cell_axis(a.x, g.inv_h, g.nc[0]);
@@ -277,9 +284,15 @@ __global__ void __launch_bounds__(256) round_kernel(const LocSet *sets, int nset
     }
     const int total = __shfl_sync(all, upto, 8);
     const int shift = from - (upto - len);   // entry number to list index
-    volatile const uint8_t *st = status;
+    volatile uint8_t *st = list_status;
+    auto settle = [&](uint8_t state) {
+        if (lane == 0) {
+            st[mine] = state;
+            status[p] = state;
+        }
+    };
     bool rejected = false, full = false;   // full: more open neighbours than the lane keeps
-    uint32_t q0 = NONE, q1 = NONE;
+    uint32_t q0 = NONE, q1 = NONE;         // places of open neighbours
     auto scan = [&]() {
         q0 = q1 = NONE;
         full = false;
@@ -291,16 +304,16 @@ __global__ void __launch_bounds__(256) round_kernel(const LocSet *sets, int nset
             const int j = e + __shfl_sync(all, shift, row);
             if (e < total) {
                 const uint32_t q = list[j];
-                const float4 b = list_pos[j];   // with q, not after it
+                const float4 b = list_pos[j];
+                const uint8_t sq = st[j];
                 if ((int64_t)q < p) {           // only higher priority
                     const float ex = a.x - b.x, ey = a.y - b.y, ez = a.z - b.z;
                     const float dist = sqrtf(ex * ex + ey * ey + ez * ez);
                     if (dist < rho * fmaxf(a.w, b.w)) {
-                        const uint8_t sq = st[q];
                         if (sq == ACCEPTED) rejected = true;
                         if (sq == UNDECIDED) {
-                            if (q0 == NONE) q0 = q;
-                            else if (q1 == NONE) q1 = q;
+                            if (q0 == NONE) q0 = (uint32_t)j;
+                            else if (q1 == NONE) q1 = (uint32_t)j;
                             else full = true;
                         }
                     }
@@ -312,11 +325,11 @@ __global__ void __launch_bounds__(256) round_kernel(const LocSet *sets, int nset
     scan();
     for (int look = 0; look < LOOKS; ++look) {
         if (__any_sync(all, rejected)) {
-            if (lane == 0) *(volatile uint8_t *)&status[p] = REJECTED;
+            settle(REJECTED);
             return;
         }
         if (!__any_sync(all, q0 != NONE || q1 != NONE)) {
-            if (lane == 0) *(volatile uint8_t *)&status[p] = ACCEPTED;
+            settle(ACCEPTED);
             return;
         }
         __nanosleep(100);
@@ -545,7 +558,7 @@ ac_status localize_many(ac_contours *const *sets, const float *E0, ac_cell *cons
     LC_CUDA(sc.cub.ensure(tmp));
     LC_CUDA(cub::DeviceRadixSort::SortPairs(sc.cub.p, tmp, ek, ek + n, sc.surv.as<int32_t>(), order, (int)n, 0,
                                             key_bits, st));
-    LC_CUDA(sc.stat.ensure(n));
+    LC_CUDA(sc.stat.ensure(2 * n));
     LC_CUDA(sc.pos.ensure(sizeof(float4) * n));
     LC_CUDA(sc.list_pos.ensure(sizeof(float4) * n));
     LC_CUDA(sc.cellk.ensure(sizeof(uint32_t) * n));
@@ -564,7 +577,8 @@ ac_status localize_many(ac_contours *const *sets, const float *E0, ac_cell *cons
     LC_CUDA(sc.cub.ensure(tmp));
     LC_CUDA(cub::DeviceScan::ExclusiveSum(sc.cub.p, tmp, start, start, (int)(ncells + 1), st));
     cell_scatter_kernel<<<blocks_for(n), 256, 0, st>>>(n, sc.cellk.as<uint32_t>(), sc.celli.as<uint32_t>(), start, pos,
-                                                       sc.list.as<uint32_t>(), sc.list_pos.as<float4>());
+                                                       sc.list.as<uint32_t>(), sc.list_pos.as<float4>(),
+                                                       sc.stat.as<uint8_t>() + n);
     count_launch();
     LC_CUDA(cudaGetLastError());
 
@@ -599,7 +613,8 @@ ac_status localize_many(ac_contours *const *sets, const float *E0, ac_cell *cons
         if (rounds > 0)
             LC_CUDA(cudaMemset2DAsync(cnt + CNT_OPEN, sizeof(int32_t) * CNT_N, 0, sizeof(int32_t), nsets, st));
         round_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(dsets, nsets, pos, n, start, sc.list.as<uint32_t>(),
-                                                              sc.list_pos.as<float4>(), status, cnt);
+                                                              sc.list_pos.as<float4>(), sc.celli.as<uint32_t>(),
+                                                              status + n, status, cnt);
         count_launch();
         LC_CUDA(cudaGetLastError());
         if (small) {
