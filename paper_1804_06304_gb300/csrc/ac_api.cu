@@ -1834,6 +1834,12 @@ extern "C" ac_status ac_autotune(ac_contours *const *sets, int32_t n_sets, ac_ev
     cudaEventCreate(&t1);
     float best_ms = 1e30f;
     TuneVal best{0, 0, {0, 0, 0}};
+    // every trial starts from the sets' own states: contours that earlier trials have moved
+    // and grown leave small halos and would make later candidates look slow
+    auto restart = [&]() {
+        for (int i = 0; i < n_sets; ++i)
+            cudaMemcpyAsync(copies[i], sets[i]->state, sizeof(float) * 5 * sets[i]->C, cudaMemcpyDeviceToDevice, st);
+    };
     for (int G : Gs) {
         for (const auto &cl : cells) {
             ac_evolve_params tp = *params;
@@ -1852,10 +1858,12 @@ extern "C" ac_status ac_autotune(ac_contours *const *sets, int32_t n_sets, ac_ev
             if (per * G / 32.0 > 16.0) continue;   // more groups than a CTA holds
             Prepared pr;
             if (prepare_sets(tsets.data(), nullptr, n_sets, &tp, nullptr, tmp[0].scratch, pr, st) != AC_OK) continue;
+            restart();
             if (enqueue_prepared(pr, tmp[0].scratch, st, nullptr, false) != AC_OK) continue;   // warm-up
             float ms = 1e30f;
             bool ok = true;
             for (int rep = 0; rep < 2 && ok; ++rep) {   // best of two timed trials
+                restart();
                 cudaEventRecord(t0, st);
                 ok = enqueue_prepared(pr, tmp[0].scratch, st, nullptr, false) == AC_OK;
                 cudaEventRecord(t1, st);
