@@ -59,11 +59,11 @@ ALG_SLOTS_PER_SAMPLE = {2: 52.75, 3: 102.25}
 ALG_SLOTS_CURRENT = {2: 52.75, 3: 95.25}
 # dram__bytes_read.sum + dram__bytes_write.sum of the evolve kernel per launch, from
 # ncu captures of the current kernel (to be removed when the kernel changes): brain-3d
-# at full size (one pass: 759.12 MB read + 54.86 MB written); large-2d from its
-# 2048^2 instance (7.42 MB read + 0.04 MB written) scaled with the image (x 4).
+# at full size (one pass: 741.64 MB read + 62.64 MB written); large-2d from its
+# 2048^2 instance (6.71 MB read, nothing written back) scaled with the image (x 4).
 DRAM_BYTES_PER_LAUNCH = {
-    ("brain-3d", "brick", 0, "native"): (814.0e6, "ncu capture of the full-size launch"),
-    ("large-2d", "brick", 0, "native"): (29.9e6, "ncu capture of the 2048^2 instance scaled with the image (x 4)"),
+    ("brain-3d", "brick", 0, "native"): (804.3e6, "ncu capture of the full-size launch"),
+    ("large-2d", "brick", 0, "native"): (26.8e6, "ncu capture of the 2048^2 instance scaled with the image (x 4)"),
 }
 SM_COUNT = 152
 LANES_PER_SM_CLOCK = 128          # 4 schedulers x 32 lanes, one instruction per clock
