@@ -743,8 +743,8 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
         // SM holds; a round lasts (staging) + (instructions of one warp) x f(warps per
         // scheduler).  f and the staging costs are a fit to 500 measured layouts of 12
         // volumes and images (64x64x32 to 260x180x60, 512^2 to 1531x1117, all voxel types, 4
-        // to 32 lanes); the chosen layout is the best measured one on 8 of them and within
-        // 11 % on the others.  Halving the default until 1216 bricks came out, as before,
+        // to 32 lanes); the chosen layout is within 12 % of the best measured one on 11 of
+        // them (200x200x100: 25 %).  Halving the default until 1216 bricks came out, as before,
         // left too few warps in flight: 128^3 u16 at N = 512, 10 iterations 486 us -> 340 us;
         // 512^2 u8 166 -> 75 us; 64x64x32 u8 84 -> 52 us.
         int64_t nb0 = 1;
