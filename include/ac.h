@@ -399,7 +399,9 @@ ac_status ac_evolve_stops(ac_contours *ctr, int64_t counts[2], void *cuda_stream
 /* Contour-iterations of the last ac_evolve / ac_evolve_batch on this handle by
  * gather path: counts[0] fast (ball inside the staged region and the volume),
  * counts[1] clamped (inside the region, crossing the volume border), counts[2]
- * global fallback (ball outside the staged region; plain path: every one).
+ * global fallback (ball outside the staged region; plain path: every one).  Contours
+ * that share a warp take the slowest path any of them needs; which ones do follows from
+ * the launch's layout alone, so the counts are the same in every run.
  * Synchronizes the stream.  Errors: AC_ERR_ARG, AC_ERR_CUDA. */
 ac_status ac_evolve_stats(ac_contours *ctr, int64_t counts[3], void *cuda_stream);
 

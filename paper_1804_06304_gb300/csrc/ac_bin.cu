@@ -2,12 +2,15 @@
 // brick kernel (arXiv:1804.06304, "Parallel Contour Evaluation": contours of one
 // image region share its voxels).
 //
-// The brick kernel needs, per brick, the list of its contours; their order within
-// the brick and the order of the bricks' lists do not matter, because contours
-// evolve independently.  So this is a counting sort without the ordering: count
+// The brick kernel needs, per brick, the list of its contours; the order of the bricks'
+// lists does not matter, because contours evolve independently.  Within a list the order
+// decides which contours share a warp, and a warp takes the slowest gather path that any
+// of its contours needs: in index order neighbours meet, and the path counters are the
+// same in every run.  So this is a counting sort without the ordering: count
 // (each contour also learns its rank in its brick), give every brick a range of the
-// list, scatter.  A brick then finds its contours with one 8-byte load (and puts a short
-// list in index order itself, while its voxels are on their way).  Bound by launch
+// list, scatter.  A brick then finds its contours with one 8-byte load, and puts a list
+// of up to LIST_MAX in index order itself, while its voxels are on their way; longer ones
+// (bricks of the caller's choice, crowded explicit seeds) are ordered here.  Bound by launch
 // latency for small sets and by the chain of dependent loads at the head of every brick
 // for large ones.  Against a radix sort by brick (five launches) and two binary searches
 // per brick, passes of 10 iterations went from 111 to 99 us (64x64x32, 2,048 contours),
@@ -47,16 +50,98 @@ __device__ __forceinline__ void clear_counts(unsigned long long *c)
     if (blockIdx.x == 0 && threadIdx.x < 3) c[threadIdx.x] = 0;
 }
 
+// A list of n > LIST_MAX contours put in index order by its block of ORDER_THREADS
+// threads: up to one contour a thread by counting the smaller ones, more through a bitmap
+// of the indices, 32 x WORDS of them at a time, with the list in order going to `tmp`
+// first.  `words` holds WORDS words, `warp_sums` 32.  Latency of one block per list:
+// 64 lists of 3,125 contours 8.4 us, 216 of 4,630 (four bitmaps) 31 us, in launches whose
+// brick kernels take 490 and 1,410 us.
+constexpr int ORDER_THREADS = 1024;
+
+template <int WORDS>
+__device__ __forceinline__ void order_list(uint32_t *list, uint32_t *tmp, uint32_t n, uint32_t *words,
+                                           uint32_t *warp_sums)
+{
+    const uint32_t t = threadIdx.x;
+    if (n <= ORDER_THREADS) {
+        if (t < n) words[t] = list[t];
+        __syncthreads();
+        if (t < n) {
+            const uint32_t g = words[t];
+            uint32_t rank = 0;
+            for (uint32_t j = 0; j < n; ++j) rank += words[j] < g ? 1 : 0;
+            list[rank] = g;
+        }
+        __syncthreads();   // `words` is free again
+        return;
+    }
+    uint32_t lo = 0xffffffffu, hi = 0;
+    for (uint32_t i = t; i < n; i += ORDER_THREADS) {
+        lo = min(lo, list[i]);
+        hi = max(hi, list[i]);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((t & 31) == 0) {
+        words[t >> 5] = lo;
+        words[32 + (t >> 5)] = hi;
+    }
+    __syncthreads();
+    for (int w = 0; w < ORDER_THREADS / 32; ++w) {
+        lo = min(lo, words[w]);
+        hi = max(hi, words[32 + w]);
+    }
+    __syncthreads();
+    constexpr int PER = WORDS / ORDER_THREADS;
+    uint32_t done = 0;
+    for (uint64_t base = lo; base <= hi; base += 32 * WORDS) {
+#pragma unroll
+        for (int j = 0; j < PER; ++j) words[j * ORDER_THREADS + t] = 0;
+        __syncthreads();
+        for (uint32_t i = t; i < n; i += ORDER_THREADS) {
+            const uint32_t g = list[i], bit = g - (uint32_t)base;
+            if (g >= base && bit < 32 * WORDS) atomicOr(&words[bit >> 5], 1u << (bit & 31));
+        }
+        __syncthreads();
+        uint32_t mine = 0, sum;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) mine += __popc(words[t * PER + j]);
+        uint32_t at = done + block_exclusive(mine, warp_sums, &sum);
+        for (int j = 0; j < PER; ++j)
+            for (uint32_t w = words[t * PER + j]; w; w &= w - 1)
+                tmp[at++] = (uint32_t)base + 32 * (t * PER + j) + (__ffs(w) - 1);
+        done += sum;
+        __syncthreads();   // `words` and `warp_sums` are free again, `tmp` is written
+    }
+    for (uint32_t i = t; i < n; i += ORDER_THREADS) list[i] = tmp[i];
+    __syncthreads();
+}
+
+// The long ones among 32 bricks, b0, b0 + step, ... (the same for the whole block)
+template <int WORDS>
+__device__ __forceinline__ void order_long_lists(const uint2 *ranges, int64_t b0, int64_t step, int64_t nb,
+                                                 uint32_t *order, uint32_t *tmp, uint32_t *words, uint32_t *warp_sums)
+{
+    const int64_t b = b0 + (int64_t)(threadIdx.x & 31) * step;
+    const uint2 mine = b < nb ? ranges[b] : make_uint2(0, 0);
+    for (unsigned todo = __ballot_sync(0xffffffffu, mine.y > LIST_MAX); todo; todo &= todo - 1) {
+        const int l = __ffs(todo) - 1;
+        const uint32_t first = __shfl_sync(0xffffffffu, mine.x, l), n = __shfl_sync(0xffffffffu, mine.y, l);
+        order_list<WORDS>(order + first, tmp + first, n, words, warp_sums);
+    }
+}
+
 // Few contours and bricks: one CTA counts in shared memory, scans and scatters, each
 // thread keeping its contours' (brick, rank) in registers: one launch instead of a clear
 // and three.  12 contours a thread is what its 64 registers hold without spills to speak of.
 __global__ void __launch_bounds__(SMALL_THREADS) bin_small_kernel(const VolDesc *vols, int n_vols, int total, int3 B,
-                                                                  int nb, uint2 *ranges, uint32_t *order,
+                                                                  int nb, uint2 *ranges, uint32_t *order, uint32_t *tmp,
                                                                   unsigned long long *path_counts)
 {
     clear_counts(path_counts);
     extern __shared__ uint32_t count[];
-    __shared__ uint32_t warp_sums[32];
+    __shared__ uint32_t warp_sums[32], words[ORDER_THREADS];
+    static_assert(SMALL_THREADS == ORDER_THREADS && SMALL_CONTOURS <= 32 * ORDER_THREADS, "one bitmap holds every index");
     for (int i = threadIdx.x; i < nb; i += SMALL_THREADS) count[i] = 0;
     __syncthreads();
     uint32_t at[SMALL_ITEMS];   // brick << 16 | rank (brick < 2^13, rank < 2^14)
@@ -76,18 +161,23 @@ __global__ void __launch_bounds__(SMALL_THREADS) bin_small_kernel(const VolDesc 
     uint32_t mine = 0, sum;
     for (int b = b0; b < b1; ++b) mine += count[b];
     uint32_t start = block_exclusive(mine, warp_sums, &sum);
+    bool any_long = false;
     for (int b = b0; b < b1; ++b) {
         const uint32_t n = count[b];
         ranges[b] = make_uint2(start, n);
         count[b] = start;
         start += n;
+        any_long = any_long || n > LIST_MAX;
     }
-    __syncthreads();
+    any_long = __syncthreads_or(any_long);
 #pragma unroll
     for (int j = 0; j < SMALL_ITEMS; ++j) {
         const int g = j * SMALL_THREADS + threadIdx.x;
         if (g < total) order[count[at[j] >> 16] + (at[j] & 0xFFFFu)] = (uint32_t)g;
     }
+    if (!any_long) return;
+    __syncthreads();
+    for (int b = 0; b < nb; b += 32) order_long_lists<ORDER_THREADS>(ranges, b, 1, nb, order, tmp, words, warp_sums);
 }
 
 __global__ void bin_count_kernel(const VolDesc *vols, int n_vols, int64_t total, int3 B, uint2 *ranges,
@@ -102,15 +192,18 @@ __global__ void bin_count_kernel(const VolDesc *vols, int n_vols, int64_t total,
     }
 }
 
-// A range of the list for every brick, in whatever order the blocks get to it.
-__global__ void __launch_bounds__(256) bin_alloc_kernel(uint2 *ranges, int64_t nb, uint32_t *cursor)
+// A range of the list for every brick, in whatever order the blocks get to it.  head[0]:
+// the list's length so far; head[1]: whether there are lists that bin_order_kernel orders.
+__global__ void __launch_bounds__(256) bin_alloc_kernel(uint2 *ranges, int64_t nb, uint32_t *head)
 {
     __shared__ uint32_t warp_sums[32], base;
     for (int64_t b0 = blockIdx.x * (int64_t)blockDim.x; b0 < nb; b0 += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = b0 + threadIdx.x;
         uint32_t sum;
-        const uint32_t off = block_exclusive(b < nb ? ranges[b].y : 0u, warp_sums, &sum);
-        if (threadIdx.x == 0) base = atomicAdd(cursor, sum);
+        const uint32_t n = b < nb ? ranges[b].y : 0u;
+        const uint32_t off = block_exclusive(n, warp_sums, &sum);
+        if (n > LIST_MAX) head[1] = 1;
+        if (threadIdx.x == 0) base = atomicAdd(&head[0], sum);
         __syncthreads();
         if (b < nb) ranges[b].x = base + off;
         __syncthreads();
@@ -122,6 +215,17 @@ __global__ void bin_scatter_kernel(const uint2 *ranges, const uint32_t *keys, co
 {
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x)
         order[ranges[keys[g]].x + ranks[g]] = (uint32_t)g;
+}
+
+// `tmp` holds a word per contour
+__global__ void __launch_bounds__(ORDER_THREADS) bin_order_kernel(const uint2 *ranges, int64_t nb, const uint32_t *head,
+                                                                  uint32_t *order, uint32_t *tmp)
+{
+    constexpr int WORDS = 8192;
+    __shared__ uint32_t words[WORDS], warp_sums[32];
+    if (head[1] == 0) return;
+    for (int64_t b = blockIdx.x; b < nb; b += 32 * (int64_t)gridDim.x)
+        order_long_lists<WORDS>(ranges, b, gridDim.x, nb, order, tmp, words, warp_sums);
 }
 
 __global__ void bin_keys_kernel(const VolDesc *vols, int n_vols, int64_t total, int3 B, uint32_t *keys,
@@ -191,7 +295,8 @@ cudaError_t launch_bin(const EvolveArgs &a, const BinSpace &s, cudaStream_t st, 
     uint2 *ranges = const_cast<uint2 *>(a.ranges);
     if (total <= SMALL_CONTOURS && bricks <= SMALL_BRICKS) {
         bin_small_kernel<<<1, SMALL_THREADS, sizeof(uint32_t) * bricks, st>>>(a.vols, a.n_vols, (int)total, B,
-                                                                              (int)bricks, ranges, s.order, a.path_counts);
+                                                                              (int)bricks, ranges, s.order, s.keys,
+                                                                              a.path_counts);
         *launches += 1;
         return cudaGetLastError();
     }
@@ -201,7 +306,10 @@ cudaError_t launch_bin(const EvolveArgs &a, const BinSpace &s, cudaStream_t st, 
                                                       a.path_counts);
     bin_alloc_kernel<<<blocks_of(bricks), 256, 0, st>>>(ranges, bricks, static_cast<uint32_t *>(s.table));
     bin_scatter_kernel<<<blocks_of(total), 256, 0, st>>>(ranges, s.keys, s.ranks, total, s.order);
-    *launches += 3;
+    // the keys have been read: their space serves the ordering
+    bin_order_kernel<<<(unsigned)std::min<int64_t>(bricks, 304), ORDER_THREADS, 0, st>>>(
+        ranges, bricks, static_cast<const uint32_t *>(s.table), s.order, s.keys);
+    *launches += 4;
     return cudaGetLastError();
 }
 

@@ -927,8 +927,6 @@ __device__ __forceinline__ int64_t lower_bound_u32(const uint32_t *keys, int64_t
 }
 
 // ----------------------------------------------------------------- brick kernel
-constexpr int LIST_MAX = 128;   // contours of a brick that are ordered by index in shared memory
-
 // One CTA per brick: TMA stages the brick plus halo into shared memory once (2D:
 // then rewritten as quads so one shared-memory load feeds a bilinear sample);
 // each group of G lanes evolves one contour of the brick through all iterations
@@ -975,7 +973,7 @@ __global__ void __maxnreg__(DIM == 2 ? 96 : 128) evolve_brick_kernel(const __gri
     // still writing shared memory when the CTA exits.  While the copy runs, the brick's
     // contours are put in increasing order (each counts the smaller ones): neighbours
     // share a warp, and with it a gather path, and the path counts do not depend on the
-    // order in which the contours were grouped.  A longer list stays as it is.
+    // order in which the contours were grouped.  A longer list arrives in order.
     __shared__ int landed;
     __shared__ uint32_t list[LIST_MAX];
     if (threadIdx.x == 0) {
