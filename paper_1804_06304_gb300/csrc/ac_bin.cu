@@ -26,8 +26,8 @@ namespace {
 
 constexpr int SMALL_THREADS = 1024;
 constexpr int SMALL_ITEMS = 12;                              // contours per thread
-constexpr int64_t SMALL_CONTOURS = SMALL_THREADS * SMALL_ITEMS;
-constexpr int64_t SMALL_BRICKS = 8192;                       // 32 KB of counters
+constexpr int SMALL_CONTOURS = SMALL_THREADS * SMALL_ITEMS;
+constexpr int SMALL_BRICKS = 8192;                           // 32 KB of counters
 
 __device__ __forceinline__ uint32_t brick_of(const VolDesc &V, int64_t k, int3 B)
 {
@@ -50,15 +50,141 @@ __device__ __forceinline__ void clear_counts(unsigned long long *c)
     if (blockIdx.x == 0 && threadIdx.x < 3) c[threadIdx.x] = 0;
 }
 
-// A list of n > LIST_MAX contours put in index order by its block of ORDER_THREADS
-// threads: up to one contour a thread by counting the smaller ones, more through a bitmap
-// of the indices, 32 x WORDS of them at a time, with the list in order going to `tmp`
-// first.  `words` holds WORDS words, `warp_sums` 32.  Latency of one block per list:
-// 64 lists of 3,125 contours 8.4 us, 216 of 4,630 (four bitmaps) 31 us, in launches whose
-// brick kernels take 490 and 1,410 us.
-constexpr int ORDER_THREADS = 1024;
+// One-CTA grouping: a list of n > LIST_MAX contours put in index order by a warp, through
+// a bitmap of the indices (all below 32 WARP_WORDS) in its own `words`; nothing to wait
+// for but the warp.  ORDER_WARPS bitmaps take the space of the counters, which have served.
+// Launches of 12,000 contours with 64 lists of 188: 90 us, with the block at one list after
+// the other 201 us, sorted 89 us; with 8 lists of 1,500: 282, 300 and 288 us.
+constexpr int WARP_WORDS = SMALL_CONTOURS / 32;
+constexpr int ORDER_WARPS = SMALL_BRICKS / WARP_WORDS;
+static_assert(SMALL_CONTOURS % 1024 == 0, "the same number of bitmap words for every lane");
 
-template <int WORDS>
+__device__ __forceinline__ void order_list_warp(uint32_t *list, uint32_t n, uint32_t *words)
+{
+    constexpr int PER = WARP_WORDS / 32;
+    const uint32_t lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) words[j * 32 + lane] = 0;
+    __syncwarp();
+    for (uint32_t i = lane; i < n; i += 32) atomicOr(&words[list[i] >> 5], 1u << (list[i] & 31));
+    __syncwarp();
+    uint32_t mine = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) mine += __popc(words[lane * PER + j]);
+    uint32_t at = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += y;
+    }
+    at -= mine;
+    for (int j = 0; j < PER; ++j)
+        for (uint32_t w = words[lane * PER + j]; w; w &= w - 1) list[at++] = 32 * (lane * PER + j) + (__ffs(w) - 1);
+    __syncwarp();   // `words` is free again
+}
+
+// Few contours and bricks: one CTA counts in shared memory, scans and scatters, each
+// thread keeping its contours' (brick, rank) in registers: one launch instead of a clear
+// and three.  12 contours a thread is what its 64 registers hold without spills to speak of.
+__global__ void __launch_bounds__(SMALL_THREADS) bin_small_kernel(const VolDesc *vols, int n_vols, int total, int3 B,
+                                                                  int nb, uint2 *ranges, uint32_t *order,
+                                                                  unsigned long long *path_counts)
+{
+    clear_counts(path_counts);
+    __shared__ uint32_t warp_sums[32], count[SMALL_BRICKS];
+    for (int i = threadIdx.x; i < nb; i += SMALL_THREADS) count[i] = 0;
+    __syncthreads();
+    uint32_t at[SMALL_ITEMS];   // brick << 16 | rank (brick < 2^13, rank < 2^14)
+#pragma unroll
+    for (int j = 0; j < SMALL_ITEMS; ++j) {
+        const int g = j * SMALL_THREADS + threadIdx.x;
+        if (g < total) {
+            const VolDesc &V = vols[find_set(vols, n_vols, g)];
+            const uint32_t b = brick_of(V, g - V.contour_base, B);
+            at[j] = b << 16 | atomicAdd(&count[b], 1u);
+        }
+    }
+    __syncthreads();
+    // thread t scans bricks [t per, (t + 1) per)
+    const int per = (nb + SMALL_THREADS - 1) / SMALL_THREADS;
+    const int b0 = threadIdx.x * per, b1 = min(b0 + per, nb);
+    uint32_t mine = 0, sum;
+    for (int b = b0; b < b1; ++b) mine += count[b];
+    uint32_t start = block_exclusive(mine, warp_sums, &sum);
+    bool any_long = false;
+    for (int b = b0; b < b1; ++b) {
+        const uint32_t n = count[b];
+        ranges[b] = make_uint2(start, n);
+        count[b] = start;
+        start += n;
+        any_long = any_long || n > LIST_MAX;
+    }
+    any_long = __syncthreads_or(any_long);
+#pragma unroll
+    for (int j = 0; j < SMALL_ITEMS; ++j) {
+        const int g = j * SMALL_THREADS + threadIdx.x;
+        if (g < total) order[count[at[j] >> 16] + (at[j] & 0xFFFFu)] = (uint32_t)g;
+    }
+    if (!any_long) return;
+    __syncthreads();
+    // warp w: the long ones among bricks w, w + ORDER_WARPS, ..., 32 of them looked at in one load
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w >= ORDER_WARPS) return;
+    for (int b = w; b < nb; b += 32 * ORDER_WARPS) {
+        const uint2 r = b + lane * ORDER_WARPS < nb ? ranges[b + lane * ORDER_WARPS] : make_uint2(0, 0);
+        for (unsigned todo = __ballot_sync(0xffffffffu, r.y > LIST_MAX); todo; todo &= todo - 1) {
+            const int l = __ffs(todo) - 1;
+            const uint32_t first = __shfl_sync(0xffffffffu, r.x, l), n = __shfl_sync(0xffffffffu, r.y, l);
+            order_list_warp(order + first, n, count + w * WARP_WORDS);
+        }
+    }
+}
+
+__global__ void bin_count_kernel(const VolDesc *vols, int n_vols, int64_t total, int3 B, uint2 *ranges,
+                                 uint32_t *keys, uint32_t *ranks, unsigned long long *path_counts)
+{
+    clear_counts(path_counts);
+    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x) {
+        const VolDesc &V = vols[find_set(vols, n_vols, g)];
+        const uint32_t b = brick_of(V, g - V.contour_base, B);
+        keys[g] = b;
+        ranks[g] = atomicAdd(&ranges[b].y, 1u);
+    }
+}
+
+// A range of the list for every brick, in whatever order the blocks get to it.  head[0]:
+// the list's length so far; head[1]: whether there are lists that bin_order_kernel orders.
+__global__ void __launch_bounds__(256) bin_alloc_kernel(uint2 *ranges, int64_t nb, uint32_t *head)
+{
+    __shared__ uint32_t warp_sums[32], base;
+    for (int64_t b0 = blockIdx.x * (int64_t)blockDim.x; b0 < nb; b0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = b0 + threadIdx.x;
+        uint32_t sum;
+        const uint32_t n = b < nb ? ranges[b].y : 0u;
+        const uint32_t off = block_exclusive(n, warp_sums, &sum);
+        if (n > LIST_MAX) head[1] = 1;
+        if (threadIdx.x == 0) base = atomicAdd(&head[0], sum);
+        __syncthreads();
+        if (b < nb) ranges[b].x = base + off;
+        __syncthreads();
+    }
+}
+
+__global__ void bin_scatter_kernel(const uint2 *ranges, const uint32_t *keys, const uint32_t *ranks, int64_t total,
+                                   uint32_t *order)
+{
+    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x)
+        order[ranges[keys[g]].x + ranks[g]] = (uint32_t)g;
+}
+
+// A list of n > LIST_MAX contours put in index order by its block: up to one contour a
+// thread by counting the smaller ones, more through a bitmap of the indices, 32 WORDS of
+// them at a time, with the list in order going to `tmp` first.  Latency of one block per
+// list: 64 lists of 3,125 contours 8.4 us, 216 of 4,630 (four bitmaps) 31 us, in launches
+// whose brick kernels take 490 and 1,410 us.
+constexpr int ORDER_THREADS = 1024;
+constexpr int WORDS = 8192;
+
 __device__ __forceinline__ void order_list(uint32_t *list, uint32_t *tmp, uint32_t n, uint32_t *words,
                                            uint32_t *warp_sums)
 {
@@ -117,115 +243,21 @@ __device__ __forceinline__ void order_list(uint32_t *list, uint32_t *tmp, uint32
     __syncthreads();
 }
 
-// The long ones among 32 bricks, b0, b0 + step, ... (the same for the whole block)
-template <int WORDS>
-__device__ __forceinline__ void order_long_lists(const uint2 *ranges, int64_t b0, int64_t step, int64_t nb,
-                                                 uint32_t *order, uint32_t *tmp, uint32_t *words, uint32_t *warp_sums)
-{
-    const int64_t b = b0 + (int64_t)(threadIdx.x & 31) * step;
-    const uint2 mine = b < nb ? ranges[b] : make_uint2(0, 0);
-    for (unsigned todo = __ballot_sync(0xffffffffu, mine.y > LIST_MAX); todo; todo &= todo - 1) {
-        const int l = __ffs(todo) - 1;
-        const uint32_t first = __shfl_sync(0xffffffffu, mine.x, l), n = __shfl_sync(0xffffffffu, mine.y, l);
-        order_list<WORDS>(order + first, tmp + first, n, words, warp_sums);
-    }
-}
-
-// Few contours and bricks: one CTA counts in shared memory, scans and scatters, each
-// thread keeping its contours' (brick, rank) in registers: one launch instead of a clear
-// and three.  12 contours a thread is what its 64 registers hold without spills to speak of.
-__global__ void __launch_bounds__(SMALL_THREADS) bin_small_kernel(const VolDesc *vols, int n_vols, int total, int3 B,
-                                                                  int nb, uint2 *ranges, uint32_t *order, uint32_t *tmp,
-                                                                  unsigned long long *path_counts)
-{
-    clear_counts(path_counts);
-    extern __shared__ uint32_t count[];
-    __shared__ uint32_t warp_sums[32], words[ORDER_THREADS];
-    static_assert(SMALL_THREADS == ORDER_THREADS && SMALL_CONTOURS <= 32 * ORDER_THREADS, "one bitmap holds every index");
-    for (int i = threadIdx.x; i < nb; i += SMALL_THREADS) count[i] = 0;
-    __syncthreads();
-    uint32_t at[SMALL_ITEMS];   // brick << 16 | rank (brick < 2^13, rank < 2^14)
-#pragma unroll
-    for (int j = 0; j < SMALL_ITEMS; ++j) {
-        const int g = j * SMALL_THREADS + threadIdx.x;
-        if (g < total) {
-            const VolDesc &V = vols[find_set(vols, n_vols, g)];
-            const uint32_t b = brick_of(V, g - V.contour_base, B);
-            at[j] = b << 16 | atomicAdd(&count[b], 1u);
-        }
-    }
-    __syncthreads();
-    // thread t scans bricks [t per, (t + 1) per)
-    const int per = (nb + SMALL_THREADS - 1) / SMALL_THREADS;
-    const int b0 = threadIdx.x * per, b1 = min(b0 + per, nb);
-    uint32_t mine = 0, sum;
-    for (int b = b0; b < b1; ++b) mine += count[b];
-    uint32_t start = block_exclusive(mine, warp_sums, &sum);
-    bool any_long = false;
-    for (int b = b0; b < b1; ++b) {
-        const uint32_t n = count[b];
-        ranges[b] = make_uint2(start, n);
-        count[b] = start;
-        start += n;
-        any_long = any_long || n > LIST_MAX;
-    }
-    any_long = __syncthreads_or(any_long);
-#pragma unroll
-    for (int j = 0; j < SMALL_ITEMS; ++j) {
-        const int g = j * SMALL_THREADS + threadIdx.x;
-        if (g < total) order[count[at[j] >> 16] + (at[j] & 0xFFFFu)] = (uint32_t)g;
-    }
-    if (!any_long) return;
-    __syncthreads();
-    for (int b = 0; b < nb; b += 32) order_long_lists<ORDER_THREADS>(ranges, b, 1, nb, order, tmp, words, warp_sums);
-}
-
-__global__ void bin_count_kernel(const VolDesc *vols, int n_vols, int64_t total, int3 B, uint2 *ranges,
-                                 uint32_t *keys, uint32_t *ranks, unsigned long long *path_counts)
-{
-    clear_counts(path_counts);
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x) {
-        const VolDesc &V = vols[find_set(vols, n_vols, g)];
-        const uint32_t b = brick_of(V, g - V.contour_base, B);
-        keys[g] = b;
-        ranks[g] = atomicAdd(&ranges[b].y, 1u);
-    }
-}
-
-// A range of the list for every brick, in whatever order the blocks get to it.  head[0]:
-// the list's length so far; head[1]: whether there are lists that bin_order_kernel orders.
-__global__ void __launch_bounds__(256) bin_alloc_kernel(uint2 *ranges, int64_t nb, uint32_t *head)
-{
-    __shared__ uint32_t warp_sums[32], base;
-    for (int64_t b0 = blockIdx.x * (int64_t)blockDim.x; b0 < nb; b0 += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = b0 + threadIdx.x;
-        uint32_t sum;
-        const uint32_t n = b < nb ? ranges[b].y : 0u;
-        const uint32_t off = block_exclusive(n, warp_sums, &sum);
-        if (n > LIST_MAX) head[1] = 1;
-        if (threadIdx.x == 0) base = atomicAdd(&head[0], sum);
-        __syncthreads();
-        if (b < nb) ranges[b].x = base + off;
-        __syncthreads();
-    }
-}
-
-__global__ void bin_scatter_kernel(const uint2 *ranges, const uint32_t *keys, const uint32_t *ranks, int64_t total,
-                                   uint32_t *order)
-{
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x)
-        order[ranges[keys[g]].x + ranks[g]] = (uint32_t)g;
-}
-
-// `tmp` holds a word per contour
+// A block looks at 32 bricks, gridDim.x apart, in one load.  `tmp` holds a word per contour.
 __global__ void __launch_bounds__(ORDER_THREADS) bin_order_kernel(const uint2 *ranges, int64_t nb, const uint32_t *head,
                                                                   uint32_t *order, uint32_t *tmp)
 {
-    constexpr int WORDS = 8192;
     __shared__ uint32_t words[WORDS], warp_sums[32];
     if (head[1] == 0) return;
-    for (int64_t b = blockIdx.x; b < nb; b += 32 * (int64_t)gridDim.x)
-        order_long_lists<WORDS>(ranges, b, gridDim.x, nb, order, tmp, words, warp_sums);
+    for (int64_t b = blockIdx.x; b < nb; b += 32 * (int64_t)gridDim.x) {
+        const int64_t mine = b + (int64_t)(threadIdx.x & 31) * gridDim.x;
+        const uint2 r = mine < nb ? ranges[mine] : make_uint2(0, 0);
+        for (unsigned todo = __ballot_sync(0xffffffffu, r.y > LIST_MAX); todo; todo &= todo - 1) {   // the same in every warp
+            const int l = __ffs(todo) - 1;
+            const uint32_t first = __shfl_sync(0xffffffffu, r.x, l), n = __shfl_sync(0xffffffffu, r.y, l);
+            order_list(order + first, tmp + first, n, words, warp_sums);
+        }
+    }
 }
 
 __global__ void bin_keys_kernel(const VolDesc *vols, int n_vols, int64_t total, int3 B, uint32_t *keys,
@@ -248,13 +280,25 @@ int key_bits(int64_t bricks)
     return b;
 }
 
+constexpr int64_t CROWDED = 512;   // contours per brick, on average
+
+bool bin_small(int64_t total, int64_t bricks) { return total <= SMALL_CONTOURS && bricks <= SMALL_BRICKS; }
+
 size_t align16(size_t n) { return (n + 15) / 16 * 16; }
 
 }  // namespace
 
 // The table of ranges costs 8 bytes and a clear per brick: not worth it when bricks
-// outnumber contours several times (a few explicit seeds in a large volume).
-bool bin_by_sort(int64_t total, int64_t bricks) { return bricks > 4 * total + 65536; }
+// outnumber contours several times (a few explicit seeds in a large volume).  Where the
+// mean list is long, counting serialises on the few bricks' counters and every list has to
+// be ordered after it.  Launches counted / sorted, in us: mean list 313 104 / 116, 438 125 /
+// 131, 602 249 / 223, 751 1083 / 1037, 1852 588 / 518, 4630 1320 / 1150.  The one-CTA form
+// counts in shared memory.
+bool bin_by_sort(int64_t total, int64_t bricks)
+{
+    const bool crowded = total > CROWDED * bricks && !bin_small(total, bricks);
+    return crowded || bricks > 4 * total + 65536;
+}
 
 cudaError_t bin_table_bytes(int64_t total, int64_t bricks, bool sort, size_t *bytes)
 {
@@ -293,10 +337,9 @@ cudaError_t launch_bin(const EvolveArgs &a, const BinSpace &s, cudaStream_t st, 
                                                key_bits(bricks), st);
     }
     uint2 *ranges = const_cast<uint2 *>(a.ranges);
-    if (total <= SMALL_CONTOURS && bricks <= SMALL_BRICKS) {
-        bin_small_kernel<<<1, SMALL_THREADS, sizeof(uint32_t) * bricks, st>>>(a.vols, a.n_vols, (int)total, B,
-                                                                              (int)bricks, ranges, s.order, s.keys,
-                                                                              a.path_counts);
+    if (bin_small(total, bricks)) {
+        bin_small_kernel<<<1, SMALL_THREADS, 0, st>>>(a.vols, a.n_vols, (int)total, B,
+                                                                              (int)bricks, ranges, s.order, a.path_counts);
         *launches += 1;
         return cudaGetLastError();
     }

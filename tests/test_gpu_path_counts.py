@@ -41,3 +41,17 @@ def test_counts_are_those_of_the_sorted_list(n, seeded, side, brick, other):
     alone = ac.ac_evolve_stats(B)
     ac.ac_evolve_batch([A, B], p)
     assert ac.ac_evolve_stats(A) == tuple(a + b for a, b in zip(counts[0], alone))
+
+
+@pytest.mark.parametrize("n,launches", [(32768, 5), (32769, 2)])
+def test_crowded_bricks_are_sorted(n, launches):
+    """64 bricks: beyond a mean list of 512 contours a sort (one kernel of the library's own, beside
+    the brick kernel) is cheaper than counting on so few counters (four)."""
+    from paper_1804_06304_gb300 import ac
+    rng = np.random.default_rng(n)
+    V = ac.ac_create_volume(rng.integers(0, 255, size=(64, 64), dtype=np.uint8))
+    seeds = np.column_stack([rng.uniform(0, 63, (n, 2)), np.zeros(n), np.ones(n)]).astype(np.float32)
+    C = ac.ac_seed(V, explicit=seeds)
+    before = ac.ac_kernel_launches()
+    ac.ac_evolve(C, ac.EvolveParams(N=64, T=1, eps0=0.0, Rmin=0.5, Rmax=1.5, brick=(8, 8, 0)))
+    assert ac.ac_kernel_launches() - before == launches
