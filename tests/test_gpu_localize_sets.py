@@ -1,0 +1,28 @@
+"""Localization of many sets in one call: the rounds take the sets in turn, their first
+survivors before what larger sets have beyond them, and find a survivor's set by a search
+of 32 sets at a time.  Every set gets the cells that it gets alone, at set counts around
+the powers of 32, with empty sets, sets without survivors, sets around a block's eight
+survivors, and sets much larger than the others."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_sets", [2, 31, 32, 33, 70, 1023, 1025])
+def test_sets_of_one_call_give_what_each_gives_alone(n_sets):
+    from paper_1804_06304_gb300 import ac
+    rng = np.random.default_rng(n_sets)
+    V = ac.ac_create_volume(np.zeros((20, 40, 60), np.uint8))
+    sizes = rng.choice([0, 1, 7, 8, 9, 40, 300], n_sets)
+    sizes[rng.integers(n_sets, size=2)] = [6000, 1500]   # far above the mean: beyond the heads
+    sets = []
+    for n in sizes:
+        c = rng.uniform(0, 1, (n, 3)) * [59, 39, 19]
+        s = ac.ac_seed(V, explicit=np.column_stack([c, rng.uniform(1.0, 5.0, n)]).astype(np.float32))
+        state = ac.ac_get_state(s)
+        state[4] = rng.uniform(-1.0, 0.3, n) if rng.random() < 0.9 else 1.0
+        ac.ac_set_state(s, state)
+        sets.append(s)
+    for got, s in zip(ac.ac_localize_batch(sets, 0.0), sets):
+        np.testing.assert_array_equal(got, ac.ac_localize(s, 0.0))
