@@ -606,10 +606,11 @@ ac_status localize_many(ac_contours *const *sets, const float *E0, ac_cell *cons
                                                      sc.celli.as<uint32_t>(), start, sc.stat.as<uint8_t>());
     count_launch();
     LC_CUDA(cudaGetLastError());
+    const uint32_t n_starts = (uint32_t)(ncells + 1);   // up to 2^31: not an int
     tmp = 0;
-    LC_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tmp, start, start, (int)(ncells + 1), st));
+    LC_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tmp, start, start, n_starts, st));
     LC_CUDA(sc.cub.ensure(tmp));
-    LC_CUDA(cub::DeviceScan::ExclusiveSum(sc.cub.p, tmp, start, start, (int)(ncells + 1), st));
+    LC_CUDA(cub::DeviceScan::ExclusiveSum(sc.cub.p, tmp, start, start, n_starts, st));
     cell_scatter_kernel<<<blocks_for(n), 256, 0, st>>>(n, sc.cellk.as<uint32_t>(), sc.celli.as<uint32_t>(), start, pos,
                                                        sc.list.as<uint32_t>(), sc.list_pos.as<float4>(),
                                                        sc.stat.as<uint8_t>() + n);

@@ -26,3 +26,25 @@ def test_sets_of_one_call_give_what_each_gives_alone(n_sets):
         sets.append(s)
     for got, s in zip(ac.ac_localize_batch(sets, 0.0), sets):
         np.testing.assert_array_equal(got, ac.ac_localize(s, 0.0))
+
+
+def test_neighbour_grids_of_2_31_minus_1_cells():
+    """The most cells one call takes (their starts are one more than an int counts): 31 sets of
+    512 x 512 x 256 cells and one of 3 x 2731 x 8191, by spacings wide against the radii."""
+    from paper_1804_06304_gb300 import ac
+    cell = float(np.float32(0.79370052598409973738)) * 1.0001
+    sets, cells = [], 0
+    for shape in [(512, 512, 256)] * 31 + [(3, 2731, 8191)]:
+        sp = tuple(float(np.float32((k - 0.5) * cell)) for k in shape)
+        V = ac.ac_create_volume(np.zeros((2, 2, 2), np.uint8), spacing=sp)
+        # two apart, one that overlaps the first, one that overlaps the last
+        c = np.array([[0, 0, 0], sp, [0.5, 0, 0], sp], np.float32) - [[0, 0, 0], [0, 0, 0], [0, 0, 0], [0.25, 0, 0]]
+        s = ac.ac_seed(V, explicit=np.column_stack([c, np.ones(4)]).astype(np.float32))
+        state = ac.ac_get_state(s)
+        state[4] = [-3.0, -1.0, -2.0, -4.0]
+        ac.ac_set_state(s, state)
+        cells += int(np.prod([int(np.floor(np.float32(w) / cell)) + 1 for w in sp], dtype=np.int64))
+        sets.append(s)
+    assert cells == 2**31 - 1
+    for got in ac.ac_localize_batch(sets, 0.0):
+        assert list(got["id"]) == [3, 0]
