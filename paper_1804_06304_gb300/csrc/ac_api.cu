@@ -680,47 +680,80 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
     // the last resort) the brick until it fits.  The staged region may take the shared
     // memory its CTA's registers leave it: in 3D (128 registers a thread) a CTA of more
     // than 8 warps has its SM alone, smaller ones share it with a second CTA.
+    auto need_of = [&](int d, int halo) {   // extent of the region along d, without padding of rows
+        int64_t need = (int64_t)B[d] + 2 * (int64_t)halo + (d == 0 ? al - 1 : 0);
+        need = std::min(need, vol->n[d] + (d == 0 ? al - 1 : 0));
+        return d == 0 ? (need + al - 1) / al * al : need;
+    };
+    // bytes of a region and its quads (2D, not for float voxels: 8-byte quads after the raw region)
+    auto quads_at = [&](int64_t raw) { return vol->ndim == 2 && vol->dtype != AC_F32 ? (raw + 127) / 128 * 128 : 0; };
+    auto bytes_of = [&](const int64_t *ext, int64_t raw) {
+        const int64_t q = quads_at(raw);
+        return q ? q + (ext[0] - 1) * (ext[1] - 1) * 8 : raw;
+    };
+    auto budget_of = [&]() -> int64_t {
+        return vol->ndim == 3 ? (warps_of() > 8 ? 215 * 1024 : 110 * 1024) : 200 * 1024;
+    };
     auto fit = [&](bool shrink_brick) {
+        int hmax = 0;
         for (int d = 0; d < vol->ndim; ++d) {
             B[d] = brick_of(d);
             h[d] = (int)std::ceil((hf * r_hint + 0.5 * p->dR) / vol->sp[d]) + 2;
+            hmax = std::max(hmax, h[d]);
         }
-        for (int iter = 0; iter < 4096; ++iter) {
-            const int64_t budget = vol->ndim == 3 ? (warps_of() > 8 ? 215 * 1024 : 110 * 1024) : 200 * 1024;
-            int64_t raw = vol->es;
+        // the least cut of the halo at which the region fits, but for padded rows (which only
+        // add), by bisection: with radii of many voxels a hundred steps for every candidate
+        auto fits_cut = [&](int cut) {
+            int64_t ext[3] = {1, 1, 1}, raw = vol->es;
+            bool box = true;
+            for (int d = 0; d < vol->ndim; ++d) {
+                ext[d] = need_of(d, std::max(1, h[d] - cut));
+                box = box && ext[d] <= 256;
+                raw *= ext[d];
+            }
+            return box && bytes_of(ext, raw) <= budget_of();
+        };
+        int lo = 0, hi = 0;
+        if (!fits_cut(0)) {
+            hi = hmax - 1;   // a halo of one voxel everywhere
+            if (!fits_cut(hi)) {
+                if (!shrink_brick) return false;
+                lo = hi;
+            }
+        }
+        while (lo < hi) {
+            const int mid = (lo + hi) / 2;
+            if (fits_cut(mid)) hi = mid; else lo = mid + 1;
+        }
+        for (int d = 0; d < vol->ndim; ++d) h[d] = std::max(1, h[d] - lo);
+        for (int iter = lo; iter < 4096; ++iter) {   // at most that many cuts in all
+            int64_t raw = vol->es, ext[3] = {1, 1, 1};
             bool fits_box = true;
             for (int d = 0; d < 3; ++d) {
-                int ext = 1;
                 if (d < vol->ndim) {
-                    int64_t need = (int64_t)B[d] + 2 * (int64_t)h[d] + (d == 0 ? al - 1 : 0);
-                    const int64_t cap = vol->n[d] + (d == 0 ? al - 1 : 0);
-                    need = std::min(need, cap);
-                    if (d == 0) need = (need + al - 1) / al * al;
+                    int64_t need = need_of(d, h[d]);
                     // 3D taps are read from the raw region: a row of a multiple of 128 bytes
                     // would put the same voxel column of every row on one shared-memory bank,
                     // so such rows get 16 more bytes (unless the region spans the volume's rows)
                     if (d == 0 && vol->ndim == 3 && need < vol->n[0] && need * vol->es % 128 == 0) need += al;
                     if (need > 256) fits_box = false;
-                    ext = (int)need;
+                    ext[d] = need;
                 }
-                pl.ext[d] = ext;
+                pl.ext[d] = (int)ext[d];
                 pl.B[d] = B[d];
                 pl.halo[d] = h[d];
-                raw *= ext;
+                raw *= ext[d];
             }
-            int64_t quad_off = 0, total = raw;
-            if (vol->ndim == 2 && vol->dtype != AC_F32) {   // 8-byte quads after the raw region
-                quad_off = (raw + 127) / 128 * 128;
-                total = quad_off + (int64_t)(pl.ext[0] - 1) * (pl.ext[1] - 1) * 8;
-            }
-            if (fits_box && total <= budget) {
+            const int64_t total = bytes_of(ext, raw);
+            if (fits_box && total <= budget_of()) {
                 pl.raw = (int)raw;
-                pl.quad_off = (int)quad_off;
+                pl.quad_off = (int)quads_at(raw);
                 pl.smem = (int)total;
                 pl.warps = warps_of();
                 return true;
             }
-            int hmax = 0, bmax = 0;
+            int bmax = 0;
+            hmax = 0;
             for (int d = 0; d < vol->ndim; ++d) {
                 hmax = std::max(hmax, h[d]);
                 bmax = std::max(bmax, B[d]);
@@ -800,12 +833,13 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
             const int *sizes = vol->ndim == 3 ? sizes3 : sizes2, n_sizes = vol->ndim == 3 ? 5 : 8;
             const int *sizes_z = vol->ndim == 3 ? sizes3 : one, n_z = vol->ndim == 3 ? 5 : 1;
             const double away = std::min(1.0, p->T / 100.0);
-            auto time_of = [&]() {   // of the current cells' fitted layout
+            auto time_of = [&](double limit) {   // of the current cells' fitted layout, if below the limit
                 // a halo cut short sends balls that have grown or moved to global memory (cut by
                 // 1.4 R0: 0.7 % of the contour-iterations of 10, 32 % of 100), and a CTA waits
                 // for its slowest warp
                 const double cut = std::max(0.0, hf - ((h[0] - 2) * (double)vol->sp[0] - 0.5 * p->dR) / r_hint);
-                return estimate(pl.warps, pl.smem) * (1.0 + away * cut * cut) * (0.915 + 0.085 * uneven());
+                const double even = estimate(pl.warps, pl.smem) * (1.0 + away * cut * cut);
+                return even * (1.0 - 1e-9) >= limit ? even : even * (0.915 + 0.085 * uneven());
             };
             // the default cells, halved until 1216 bricks come out: kept unless another layout
             // promises 7 % (what the estimate is good for)
@@ -820,7 +854,7 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
                 for (int d = 0; d < vol->ndim; ++d) nb *= (vol->n[d] + brick_of(d) - 1) / brick_of(d);
             }
             int chosen[3] = {cells[0], cells[1], cells[2]};
-            double best = fit(false) ? 0.93 * time_of() : 1e300;
+            double best = fit(false) ? 0.93 * time_of(1e300) : 1e300;
             for (int z = 0; z < n_z; ++z)
                 for (int y = 0; y < n_sizes; ++y)
                     for (int x = 0; x < n_sizes; ++x) {
@@ -830,7 +864,7 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
                         if (cells[0] * cells[1] * cells[2] * G > 16 * 32) continue;
                         for (int d = 0; d < vol->ndim; ++d) B[d] = brick_of(d);
                         if (estimate(warps_of(), 0) >= best || !fit(false)) continue;   // without staging: a lower bound
-                        const double t = time_of();
+                        const double t = time_of(best);
                         if (t < best) {
                             best = t;
                             for (int d = 0; d < 3; ++d) chosen[d] = cells[d];
@@ -844,7 +878,7 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
 }
 
 // plan_evolve, or the plan of the owner's last launch when nothing that it depends on
-// has changed (a search over bricks costs about 20 us of host time).
+// has changed (a search over bricks costs up to 13 us of host time).
 ac_status plan_with_memo(const ac_volume *vol, double stride_hint, double r_hint, const ac_evolve_params *p,
                          PlanMemo &memo, Plan &pl)
 {
@@ -1448,7 +1482,8 @@ extern "C" ac_status ac_evolve_static(const void *volume_dev, ac_dtype dtype, in
     ctr.r_hint = r0;
     ctr.stride_hint = stride;
     Plan pl;
-    s = plan_evolve(&vol, stride, r0, p, pl);
+    static thread_local PlanMemo memo;   // there is no handle to keep it in
+    s = plan_with_memo(&vol, stride, r0, p, memo, pl);
     if (s != AC_OK) return s;
 
     EvolveArgs a;
