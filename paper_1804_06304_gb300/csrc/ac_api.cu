@@ -817,7 +817,7 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
                     full *= std::min(std::max(1.0, std::floor(vol->n[d] * (double)vol->sp[d] / stride_hint)),
                                      std::ceil(cell - 1e-6));
                 }
-                const int r = std::max(1, std::min({reg_warps / warps, 233472 / (smem + 1088), 32}));
+                const int r = std::max(1, std::min({reg_warps / warps, SM_SMEM / (smem + BRICK_SMEM_EXTRA), 32}));
                 const double busy = std::min(lattice / nb / per_warp, (double)warps);   // warps at work, on average
                 const double most = std::min((double)warps, std::ceil(full / per_warp));
                 const double passes = std::ceil(full / per_warp / warps);

@@ -976,6 +976,7 @@ __global__ void __maxnreg__(DIM == 2 ? 96 : 128) evolve_brick_kernel(const __gri
     // order in which the contours were grouped.  A longer list arrives in order.
     __shared__ int landed;
     __shared__ uint32_t list[LIST_MAX];
+    static_assert(sizeof(mbar) + sizeof(landed) + sizeof(list) <= BRICK_SMEM_EXTRA - 1024, "what the planner counts");
     if (threadIdx.x == 0) {
         mbar_init(&mbar, 1);
         mbar_expect_tx(&mbar, (uint32_t)a.raw_bytes);
