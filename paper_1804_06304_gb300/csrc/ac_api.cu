@@ -612,8 +612,10 @@ ac_status check_params(const ac_evolve_params *p)
 // outgrow it read from global memory for that iteration).  A region starts at max(0, brick - halo)
 // (x rounded down to the 16-byte TMA alignment) and never extends past what the
 // volume needs; when the region would exceed the shared-memory budget the halo,
-// then the brick, shrinks.
-ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, const ac_evolve_params *p, Plan &pl)
+// then the brick, shrinks.  `vol`: the geometry to plan for (see launch_geometry), `sets`:
+// all volumes of the launch, which share one layout.
+ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets, double stride_hint, double r_hint,
+                      const ac_evolve_params *p, Plan &pl)
 {
     pl.brick = p->path == AC_PATH_BRICK;
     pl.grid = p->path == AC_PATH_GRID;
@@ -768,9 +770,44 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
         }
         return false;
     };
+    auto lattice_along = [&](const SetGeometry &g, int d) {
+        return std::max(1.0, std::floor(g.n[d] * (double)g.sp[d] / stride_hint));
+    };
+    // Every volume's bricks and, along a full brick, lattice contours: kept per axis and brick
+    // size, because a launch may have many volumes and the search tries many bricks.
+    const size_t n_geo = sets.size();
+    std::vector<double> counted[3];   // per size: n_geo numbers of bricks, n_geo of contours
+    std::vector<int> sizes_of[3];
+    auto along = [&](int d) -> const double * {
+        size_t k = 0;
+        while (k < sizes_of[d].size() && sizes_of[d][k] != B[d]) ++k;
+        if (k == sizes_of[d].size()) {
+            sizes_of[d].push_back(B[d]);
+            counted[d].resize(2 * n_geo * (k + 1));
+            double *t = &counted[d][2 * n_geo * k];
+            for (size_t i = 0; i < n_geo; ++i) {
+                const SetGeometry &g = sets[i];
+                t[i] = d < vol->ndim ? (double)((g.n[d] + B[d] - 1) / B[d]) : 1.0;
+                t[n_geo + i] = d < vol->ndim ? std::min(lattice_along(g, d), std::ceil(B[d] * (double)g.sp[d] / stride_hint - 1e-6)) : 1.0;
+            }
+        }
+        return &counted[d][2 * n_geo * k];
+    };
+    auto count_bricks = [&]() {   // of the launch, for the current B
+        const double *x = along(0), *y = along(1), *z = along(2);
+        double nb = 0.0;
+        for (size_t i = 0; i < n_geo; ++i) nb += sets[i].count * x[i] * y[i] * z[i];
+        return nb;
+    };
+    auto full_brick = [&]() {     // the most contours that a brick holds
+        const double *x = along(0) + n_geo, *y = along(1) + n_geo, *z = along(2) + n_geo;
+        double full = 1.0;
+        for (size_t i = 0; i < n_geo; ++i) full = std::max(full, x[i] * y[i] * z[i]);
+        return full;
+    };
     for (int d = 0; d < vol->ndim; ++d) B[d] = brick_of(d);
     if (own_bricks) {
-        // A volume of fewer than 1216 default bricks (four per slot, two slots on each of
+        // A launch of fewer than 1216 default bricks (four per slot, two slots on each of
         // 152 SMs) leaves SMs idle or ends in a nearly empty wave.  Its bricks are chosen by
         // an estimate of the launch's time in SM cycles: CTAs run in rounds of as many as an
         // SM holds; a round lasts (staging) + (instructions of one warp) x f(warps per
@@ -779,14 +816,25 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
         // to 32 lanes); the chosen layout is within 12 % of the best measured one on 11 of
         // them (200x200x100: 25 %).  Halving the default until 1216 bricks came out, as before,
         // left too few warps in flight: 128^3 u16 at N = 512, 10 iterations 486 us -> 340 us;
-        // 512^2 u8 166 -> 75 us; 64x64x32 u8 84 -> 52 us.
-        int64_t nb0 = 1;
-        double lattice = 1.0;
-        for (int d = 0; d < vol->ndim; ++d) {
-            nb0 *= (vol->n[d] + B[d] - 1) / B[d];
-            lattice *= std::max(1.0, std::floor(vol->n[d] * (double)vol->sp[d] / stride_hint));
+        // 512^2 u8 166 -> 75 us; 64x64x32 u8 84 -> 52 us.  A launch over several volumes is
+        // estimated as one, and as soon as one of them would be small alone (10 iterations
+        // with the default bricks, in us: 60 volumes of 64x64x32 757 -> 608, 64^3 to
+        // 512x512x128 4137 -> 2773, 16 of 30 to 300 voxels a side 8,930 -> 5,610); volumes
+        // that all have 1216 bricks keep the default.
+        const double nb0 = count_bricks();
+        bool small = nb0 < 1216;
+        for (const SetGeometry &g : sets) {
+            double nb = 1.0;
+            for (int d = 0; d < vol->ndim; ++d) nb *= (double)((g.n[d] + B[d] - 1) / B[d]);
+            small = small || nb < 1216;
         }
-        if (nb0 < 1216) {
+        if (small) {
+            double lattice = 0.0;
+            for (const SetGeometry &g : sets) {
+                double one = (double)g.count;
+                for (int d = 0; d < vol->ndim; ++d) one *= lattice_along(g, d);
+                lattice += one;
+            }
             const int reg_warps = vol->ndim == 3 ? 16 : 21;   // warps an SM's registers hold
             const double per_warp = 32.0 / G;                 // contours a warp evolves at once
             const double instr = p->T * ((double)p->N / G * (vol->ndim == 3 ? 115.0 : 85.0) + 400.0);
@@ -810,13 +858,7 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
                 return 32.0 * sq / (sum * sum);
             };
             auto estimate = [&](int warps, int smem) {
-                double nb = 1.0, full = 1.0;   // bricks; contours of a full brick
-                for (int d = 0; d < vol->ndim; ++d) {
-                    const double cell = B[d] * (double)vol->sp[d] / stride_hint;
-                    nb *= (double)((vol->n[d] + B[d] - 1) / B[d]);
-                    full *= std::min(std::max(1.0, std::floor(vol->n[d] * (double)vol->sp[d] / stride_hint)),
-                                     std::ceil(cell - 1e-6));
-                }
+                const double nb = count_bricks(), full = full_brick();
                 const int r = std::max(1, std::min({reg_warps / warps, SM_SMEM / (smem + BRICK_SMEM_EXTRA), 32}));
                 const double busy = std::min(lattice / nb / per_warp, (double)warps);   // warps at work, on average
                 const double most = std::min((double)warps, std::ceil(full / per_warp));
@@ -844,14 +886,14 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
             // the default cells, halved until 1216 bricks come out: kept unless another layout
             // promises 7 % (what the estimate is good for)
             const int min_cells = vol->ndim == 3 ? 1 : 2;
-            for (int64_t nb = nb0; nb < 1216;) {
+            for (double nb = nb0; nb < 1216;) {
                 int dm = -1;
                 for (int d = 0; d < vol->ndim; ++d)
                     if (cells[d] > min_cells && (dm < 0 || cells[d] > cells[dm])) dm = d;
                 if (dm < 0) break;
                 cells[dm] = std::max(min_cells, cells[dm] / 2);
-                nb = 1;
-                for (int d = 0; d < vol->ndim; ++d) nb *= (vol->n[d] + brick_of(d) - 1) / brick_of(d);
+                B[dm] = brick_of(dm);
+                nb = count_bricks();
             }
             int chosen[3] = {cells[0], cells[1], cells[2]};
             double best = fit(false) ? 0.93 * time_of(1e300) : 1e300;
@@ -877,10 +919,57 @@ ac_status plan_evolve(const ac_volume *vol, double stride_hint, double r_hint, c
     AC_FAIL(AC_ERR_ARG, "ac_evolve: staged region cannot fit the shared-memory budget; use smaller bricks");
 }
 
+// The geometry that a launch over several volumes is planned for: every axis as long as the
+// longest of them, with the spacing of the volume with the most lattice contours, whatever
+// the order of the sets.  Planned for the first volume alone, a launch over 30 volumes of
+// 128^3 behind one of 40x40x20 took 74.9 ms (that volume's bricks and regions), in the
+// opposite order 7.4 ms.
+void launch_geometry(ac_contours *const *sets, int n_sets, double stride_hint, ac_volume &vol,
+                     std::vector<SetGeometry> &all)
+{
+    vol = *sets[0]->vol;   // voxel type and dimensions are common
+    all.clear();
+    double most = -1.0;
+    for (int i = 0; i < n_sets; ++i) {
+        const ac_volume *v = sets[i]->vol;
+        SetGeometry g;
+        std::memset(&g, 0, sizeof(g));
+        g.count = 1;
+        double lattice = 1.0;
+        for (int d = 0; d < 3; ++d) {
+            g.n[d] = v->n[d];
+            g.sp[d] = v->sp[d];
+            vol.n[d] = std::max(vol.n[d], v->n[d]);
+            if (d < v->ndim) lattice *= std::max(1.0, std::floor(v->n[d] * (double)v->sp[d] / stride_hint));
+        }
+        if (lattice > most || (lattice == most && std::lexicographical_compare(vol.sp, vol.sp + 3, g.sp, g.sp + 3))) {
+            most = lattice;
+            for (int d = 0; d < 3; ++d) vol.sp[d] = g.sp[d];
+        }
+        if (!all.empty() && std::memcmp(all.back().n, g.n, sizeof(g.n)) == 0 &&
+            std::memcmp(all.back().sp, g.sp, sizeof(g.sp)) == 0)
+            ++all.back().count;
+        else
+            all.push_back(g);
+    }
+}
+
+std::vector<SetGeometry> one_volume(const ac_volume &v)
+{
+    SetGeometry g;
+    std::memset(&g, 0, sizeof(g));
+    for (int d = 0; d < 3; ++d) {
+        g.n[d] = v.n[d];
+        g.sp[d] = v.sp[d];
+    }
+    g.count = 1;
+    return {g};
+}
+
 // plan_evolve, or the plan of the owner's last launch when nothing that it depends on
-// has changed (a search over bricks costs up to 13 us of host time).
-ac_status plan_with_memo(const ac_volume *vol, double stride_hint, double r_hint, const ac_evolve_params *p,
-                         PlanMemo &memo, Plan &pl)
+// has changed (a search over bricks costs up to 13 us of host time for one volume).
+ac_status plan_with_memo(const ac_volume *vol, std::vector<SetGeometry> &&sets, double stride_hint, double r_hint,
+                         const ac_evolve_params *p, PlanMemo &memo, Plan &pl)
 {
     PlanKey key;
     std::memset(&key, 0, sizeof(key));
@@ -902,14 +991,17 @@ ac_status plan_with_memo(const ac_volume *vol, double stride_hint, double r_hint
     key.sampling = p->sampling;
     key.dR = p->dR;
     key.halo_factor = p->halo_factor;
-    if (memo.valid && std::memcmp(&memo.key, &key, sizeof(key)) == 0) {
+    const size_t bytes = sizeof(SetGeometry) * sets.size();   // zeroed before they were filled in
+    if (memo.valid && std::memcmp(&memo.key, &key, sizeof(key)) == 0 && memo.sets.size() == sets.size() &&
+        std::memcmp(memo.sets.data(), sets.data(), bytes) == 0) {
         pl = memo.plan;
         return AC_OK;
     }
     memo.valid = false;
-    const ac_status s = plan_evolve(vol, stride_hint, r_hint, p, pl);
+    const ac_status s = plan_evolve(vol, sets, stride_hint, r_hint, p, pl);
     if (s != AC_OK) return s;
     memo.key = key;
+    memo.sets = std::move(sets);
     memo.plan = pl;
     memo.valid = true;
     return AC_OK;
@@ -1073,7 +1165,10 @@ ac_status prepare_sets(ac_contours *const *sets, const ac_batch_item *items, int
         return AC_OK;
     }
     Plan &pl = pr.pl;
-    s = plan_with_memo(v0, stride_hint, r_hint, p, sc.memo, pl);
+    ac_volume common;
+    std::vector<SetGeometry> geometry;
+    launch_geometry(sets, n_sets, stride_hint, common, geometry);
+    s = plan_with_memo(&common, std::move(geometry), stride_hint, r_hint, p, sc.memo, pl);
     if (s != AC_OK) return s;
     pr.dtype = v0->dtype;
     pr.n_sets = n_sets;
@@ -1392,7 +1487,7 @@ extern "C" ac_status ac_plan_layout(int32_t ndim, ac_dtype dtype, const int64_t 
     vol.pitch_y = vol.n[0];
     vol.pitch_z = vol.n[0] * vol.n[1];
     Plan pl;
-    s = plan_evolve(&vol, stride, r0, p, pl);
+    s = plan_evolve(&vol, one_volume(vol), stride, r0, p, pl);
     if (s != AC_OK) return s;
     std::memset(out, 0, sizeof(*out));
     out->lanes_per_contour = pl.G;
@@ -1483,7 +1578,7 @@ extern "C" ac_status ac_evolve_static(const void *volume_dev, ac_dtype dtype, in
     ctr.stride_hint = stride;
     Plan pl;
     static thread_local PlanMemo memo;   // there is no handle to keep it in
-    s = plan_with_memo(&vol, stride, r0, p, memo, pl);
+    s = plan_with_memo(&vol, one_volume(vol), stride, r0, p, memo, pl);
     if (s != AC_OK) return s;
 
     EvolveArgs a;

@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <string>
+#include <vector>
 
 #include "ac_internal.cuh"
 
@@ -96,9 +97,16 @@ struct PlanKey {
     float sp[3], dR, halo_factor;
     int dtype, ndim, N, T, path, lanes, comp, warps, sampling, brick[3];
 };
+// Volumes of one geometry among a launch's sets
+struct SetGeometry {
+    int64_t n[3];
+    float sp[3];
+    int64_t count;
+};
 struct PlanMemo {
     bool valid = false;
     PlanKey key;
+    std::vector<SetGeometry> sets;
     Plan plan;
 };
 
