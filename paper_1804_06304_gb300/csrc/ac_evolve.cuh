@@ -100,14 +100,7 @@ __device__ __forceinline__ void iter_consts(IterC<DIM> &ic, const float *c, floa
 
 // Fast path: every tap of the ball lies inside the volume and the staged region,
 // so no clamping; floor and index come from one add rounded toward minus infinity
-// onto 2^23 + (ci - region origin).
-__device__ __forceinline__ void fast_axis(float x, float M, int &idx, float &fr)
-{
-    const float t = add_rd(x, M);
-    fr = x - (t - M);
-    idx = (int)__float_as_uint(t) - 0x4B000000;
-}
-// the same for the x and y axes in packed pairs
+// onto 2^23 + (ci - region origin).  The x and y axes in packed pairs.
 __device__ __forceinline__ void fast_axes2(float2 x, float2 M, int &i0, int &i1, float2 &fr)
 {
     const float2 t = __fadd2_rd(x, M);
@@ -232,19 +225,15 @@ template <typename QT, bool DIFF> struct QuadFast {
     }
     __device__ __forceinline__ float2 at2(float2 x0, float2 x1) const
     {
-#ifdef AC_CHECKED
-        return at_each(*this, x0, x1);
-#else
         constexpr float Z = QuadBias<QT>::value;
         const FastIndex2 t(x0, x1, M0, M[1], pitch);
-        const float4 a = quad_f(lds_quad<QT>(C + (uint32_t)sizeof(QT) * __float_as_uint(t.i.x)));
-        const float4 b = quad_f(lds_quad<QT>(C + (uint32_t)sizeof(QT) * __float_as_uint(t.i.y)));
+        const float4 a = quad_f(lds_quad<QT>(checked_lds(C + (uint32_t)sizeof(QT) * __float_as_uint(t.i.x), 0, Q, nq, st)));
+        const float4 b = quad_f(lds_quad<QT>(checked_lds(C + (uint32_t)sizeof(QT) * __float_as_uint(t.i.y), 0, Q, nq, st)));
         const float2 v0 = make_float2(a.x, b.x), v1 = make_float2(a.y, b.y);
         const float2 e0 = make_float2(a.z, b.z), e1 = make_float2(a.w, b.w);
         const float2 r0 = fma2(t.f0, DIFF ? e0 : sub2(e0, v0), Z != 0.0f ? sub2(v0, dup2(Z)) : v0);   // row y0 at x
         const float2 r1 = fma2(t.f0, DIFF ? e1 : sub2(e1, v1), Z != 0.0f ? sub2(v1, dup2(Z)) : v1);   // row y1
         return fma2(t.f1, sub2(r1, r0), r0);
-#endif
     }
 };
 
@@ -304,26 +293,7 @@ template <typename T> struct GlobalLoad {
     }
 };
 
-template <int DIM, typename T> struct RawFast {
-    const T *p;
-    int py, pz;
-    float M[3];
-    int64_t n;       // voxels in the region (checked build)
-    int32_t *st;
-    __device__ __forceinline__ float at(float x0, float x1, float x2) const
-    {
-        int i0, i1, i2 = 0;
-        float2 fr;
-        float f2 = 0.0f;
-        fast_axes2(make_float2(x0, x1), make_float2(M[0], M[1]), i0, i1, fr);
-        if (DIM == 3) fast_axis(x2, M[2], i2, f2);
-        return interp<DIM, T>(p + i0 + i1 * py + i2 * pz, py, pz, fr.x, fr.y, f2, SmemLoad<T>{p, n, st});
-    }
-    __device__ __forceinline__ float2 at2(float2 x0, float2 x1) const { return at_each(*this, x0, x1); }
-};
-
-// Raw taps through 32-bit shared-memory addresses (3D fast path; the bounds-checked
-// build keeps RawFast): the directed
+// Raw taps through 32-bit shared-memory addresses (3D): the directed
 // add leaves bits(t_d) = 2^23 + tap index d (as an integer 0x4B000000 + index), so the
 // byte address of the base tap is C + es bits(t0) + es py bits(t1) + es pz bits(t2)
 // with the biases folded into C (arithmetic modulo 2^32); the other taps are
@@ -385,6 +355,9 @@ template <> __device__ __forceinline__ float lds_tap_next<float>(uint32_t a)
 // four contours take it for 12 % of the contour-iterations of 512x512x128 (10 iterations
 // 6.62 -> 6.44 ms) and 37 % of 128^3 (338 -> 324 us).
 template <typename T, bool CLAMP> struct RawFast3S {
+    const T *p;          // the region, its voxels and the status word (checked build)
+    int64_t n;
+    int32_t *st;
     uint32_t C;          // folded base address (see above)
     uint32_t pyb, pzb;   // row and plane pitch, bytes
     float M[3];          // 2^23 + index of the centre voxel, per axis
@@ -406,7 +379,8 @@ template <typename T, bool CLAMP> struct RawFast3S {
         }
         const float2 fr = sub2(make_float2(x0, x1), sub2(t, make_float2(M[0], M[1])));
         const float f2 = x2 - (t2 - M[2]);
-        const uint32_t a = C + es * __float_as_uint(t.x) + pyb * __float_as_uint(t.y) + pzb * __float_as_uint(t2);
+        const uint32_t a = checked_lds(C + es * __float_as_uint(t.x) + pyb * __float_as_uint(t.y) + pzb * __float_as_uint(t2),
+                                       es + pyb + pzb, p, n, st);
         const uint32_t r = a + pzb, ay = a + pyb, ry = r + pyb;
         const float2 lo0 = make_float2(lds_tap<T>(a), lds_tap<T>(r)), hi0 = make_float2(lds_tap_next<T>(a), lds_tap_next<T>(r));
         const float2 lo1 = make_float2(lds_tap<T>(ay), lds_tap<T>(ry)), hi1 = make_float2(lds_tap_next<T>(ay), lds_tap_next<T>(ry));
@@ -419,19 +393,27 @@ template <typename T, bool CLAMP> struct RawFast3S {
 
 // The 2D fast path without quads: four taps a sample, two samples at once.
 template <typename T> struct RawFast2S {
-    RawFast<2, T> one;
+    const T *p;
+    int py;              // elements per row
+    float M[2];          // 2^23 + index of the centre voxel, per axis
+    int64_t n;           // voxels in the region (checked build)
+    int32_t *st;
     uint32_t C, pyb;     // address of the region, biases folded (modulo 2^32); row pitch, bytes
     float M0, pitch;     // 2^23 + linear index of the centre voxel; elements per row
-    __device__ __forceinline__ float at(float x0, float x1, float x2) const { return one.at(x0, x1, x2); }
+    __device__ __forceinline__ float at(float x0, float x1, float) const
+    {
+        int i0, i1;
+        float2 fr;
+        fast_axes2(make_float2(x0, x1), make_float2(M[0], M[1]), i0, i1, fr);
+        return interp<2, T>(p + i0 + i1 * py, py, 0, fr.x, fr.y, 0.0f, SmemLoad<T>{p, n, st});
+    }
     __device__ __forceinline__ float2 at2(float2 x0, float2 x1) const
     {
-#ifdef AC_CHECKED
-        return at_each(one, x0, x1);
-#else
         constexpr float Z = TapBias<T>::value;
-        const FastIndex2 t(x0, x1, M0, one.M[1], pitch);
-        const uint32_t a = C + (uint32_t)sizeof(T) * __float_as_uint(t.i.x);
-        const uint32_t b = C + (uint32_t)sizeof(T) * __float_as_uint(t.i.y);
+        const FastIndex2 t(x0, x1, M0, M[1], pitch);
+        const uint32_t far = (uint32_t)sizeof(T) + pyb;
+        const uint32_t a = checked_lds(C + (uint32_t)sizeof(T) * __float_as_uint(t.i.x), far, p, n, st);
+        const uint32_t b = checked_lds(C + (uint32_t)sizeof(T) * __float_as_uint(t.i.y), far, p, n, st);
         auto row = [&](uint32_t p, uint32_t q) {
             const float2 lo = make_float2(lds_tap<T>(p), lds_tap<T>(q));
             const float2 hi = make_float2(lds_tap_next<T>(p), lds_tap_next<T>(q));
@@ -439,32 +421,30 @@ template <typename T> struct RawFast2S {
         };
         const float2 r0 = row(a, b), r1 = row(a + pyb, b + pyb);
         return fma2(t.f1, sub2(r1, r0), r0);
-#endif
     }
 };
 
-// Clamped path in shared memory (quads in 2D, raw voxels otherwise).
-template <int DIM, typename T, bool QUAD> struct SmemClamp {
+// Clamped path in shared memory, 2D (quads, or raw voxels where there are none).
+template <typename T, bool QUAD> struct SmemClamp {
     const void *p;
-    int py, pz;      // raw pitches, or quads per row in py
-    AxisSplit ax[3];
-    int o[3];        // centre voxel relative to the region origin
+    int py;          // quads or voxels per row
+    AxisSplit ax[2];
+    int o[2];        // centre voxel relative to the region origin
     int64_t n;       // quads or voxels in the region (checked build)
     int32_t *st;
-    __device__ __forceinline__ float at(float x0, float x1, float x2) const
+    __device__ __forceinline__ float at(float x0, float x1, float) const
     {
-        int b0, b1, b2 = 0;
-        float f0, f1, f2 = 0.0f;
+        int b0, b1;
+        float f0, f1;
         axis_tap(ax[0], x0, b0, f0);
         axis_tap(ax[1], x1, b1, f1);
-        if (DIM == 3) axis_tap(ax[2], x2, b2, f2);
         if (QUAD) {
             using QT = typename QuadOf<T>::type;
             const int64_t qi = checked((int64_t)(o[1] + b1) * py + (o[0] + b0), n, st);
             return quad_lerp<QT, QuadOf<T>::diff>(reinterpret_cast<const QT *>(p)[qi], f0, f1);
         }
-        const T *q = reinterpret_cast<const T *>(p) + (o[0] + b0) + (o[1] + b1) * py + (DIM == 3 ? (o[2] + b2) * pz : 0);
-        return interp<DIM, T>(q, py, pz, f0, f1, f2, SmemLoad<T>{reinterpret_cast<const T *>(p), n, st});
+        const T *q = reinterpret_cast<const T *>(p) + (o[0] + b0) + (o[1] + b1) * py;
+        return interp<2, T>(q, py, 0, f0, f1, 0.0f, SmemLoad<T>{reinterpret_cast<const T *>(p), n, st});
     }
     __device__ __forceinline__ float2 at2(float2 x0, float2 x1) const { return at_each(*this, x0, x1); }
 };
@@ -1125,32 +1105,24 @@ __global__ void __maxnreg__(DIM == 2 ? 96 : 128) evolve_brick_kernel(const __gri
                                                       8388608.0f + (float)(o[0] + o[1] * qp), (float)qp};
                     s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
                 } else if constexpr (DIM == 2) {
-                    RawFast2S<T> gat{{reg, py, pz, {M[0], M[1], M[2]}, nraw, V.status}, raw_C, (uint32_t)(sizeof(T) * py),
+                    RawFast2S<T> gat{reg, py, {M[0], M[1]}, nraw, V.status, raw_C, (uint32_t)(sizeof(T) * py),
                                      8388608.0f + (float)(o[0] + o[1] * py), (float)py};
                     s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
                 } else {
-#ifndef AC_CHECKED
-                    // 32-bit shared addresses, biases folded into raw_C
-                    RawFast3S<T, false> gat{raw_C, (uint32_t)(sizeof(T) * py), (uint32_t)(sizeof(T) * pz),
-                                            {M[0], M[1], M[2]}, {}, {}};
-#else
-                    RawFast<DIM, T> gat{reg, py, pz, {M[0], M[1], M[2]}, nraw, V.status};
-#endif
+                    RawFast3S<T, false> gat{reg, nraw, V.status, raw_C, (uint32_t)(sizeof(T) * py),
+                                            (uint32_t)(sizeof(T) * pz), {M[0], M[1], M[2]}, {}, {}};
                     s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
                 }
             } else if (use_smem) {
-#ifndef AC_CHECKED
                 if constexpr (DIM == 3) {
-                    RawFast3S<T, true> gat{raw_C, (uint32_t)(sizeof(T) * py), (uint32_t)(sizeof(T) * pz),
-                                           {M[0], M[1], M[2]}, {ic.ax[0].lo, ic.ax[1].lo, ic.ax[2].lo},
+                    RawFast3S<T, true> gat{reg, nraw, V.status, raw_C, (uint32_t)(sizeof(T) * py),
+                                           (uint32_t)(sizeof(T) * pz), {M[0], M[1], M[2]},
+                                           {ic.ax[0].lo, ic.ax[1].lo, ic.ax[2].lo},
                                            {ic.ax[0].hi, ic.ax[1].hi, ic.ax[2].hi}};
                     s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
-                } else
-#endif
-                {
-                    SmemClamp<DIM, T, quad> gat{quad ? (const void *)Q : (const void *)reg, quad ? qp : py,
-                                                quad ? 0 : pz, {ic.ax[0], ic.ax[1], ic.ax[2]}, {o[0], o[1], o[2]},
-                                                quad ? (int64_t)nquads : nraw, V.status};
+                } else {
+                    SmemClamp<T, quad> gat{quad ? (const void *)Q : (const void *)reg, quad ? qp : py,
+                                           {ic.ax[0], ic.ax[1]}, {o[0], o[1]}, quad ? (int64_t)nquads : nraw, V.status};
                     s = eval_contour<DIM, G, COMP, ACC>(gat, ic, R, a, n, (uint32_t)k, V.stream, V.scale, lig, mask);
                 }
             } else {
