@@ -23,9 +23,52 @@
 namespace ac {
 namespace {
 
-template <int DIM, typename T, int G, bool COMP>
+// Whether the roots and quotients of an evaluation with radius R are Newton steps.  Voxels
+// nearer to the centre than the root of ROOT_MIN have a root that is only near enough: they
+// must lie inside both bands, where the root plays no part.  Squared distances, also of the
+// voxel beside a chord's last, and (integer voxels) k I stay within the ranges of sqrt2 and
+// div2.  What remains (spacings below about 1e-14 or above 1e7, radii below half a band)
+// takes the operations for any operand; there a chord of ROOT_MIN's root would be
+// thousands of voxels long.
+__device__ __forceinline__ bool newton_range(const EvolveArgs &a, const VolDesc &V, float R)
+{
+    constexpr float NEAR = 7.105427357601002e-15f;   // 2^-47
+    const float Ro = R + 0.5f * a.dR, Ro2 = __fmul_rn(Ro, Ro);
+    const float kmin = fminf(fabsf(a.kr1), fabsf(a.kr2)), kmax = fmaxf(fabsf(a.kr1), fabsf(a.kr2));
+    return Ro2 > 8.470329472543003e-22f && Ro2 < 1.125899906842624e15f &&   // 2^-70, 2^50
+           V.sp[0] < 33554432.0f &&                                         // 2^25
+           fmaf(-a.rho * R + NEAR, a.inv_dr, 0.5f) < -0.001f && fmaf(NEAR - R, a.inv_dR, 0.5f) < -0.001f &&
+           kmin > 9.094947017729282e-13f && kmax < 1.099511627776e12f;      // 2^-40, 2^40
+}
+
+// Whether div2 was right for all numerators of a ball, known after it (`s`: the evaluation).
+// Integer voxels cannot leave its range.  binary16: none infinite or NaN, which leave no
+// finite energy.  float: by the largest numerator.  (Numerators below QUOTIENT_MIN have an
+// error in their last place: 2^-48 of the largest one is where the compensated sums end, so
+// that one has to be 2^24 above.)
+template <typename T> struct Numerators {
+    __device__ __forceinline__ void add(float2) {}
+    template <int G> __device__ __forceinline__ bool fine(const Step &, unsigned) const { return true; }
+};
+template <> struct Numerators<__half> {
+    __device__ __forceinline__ void add(float2) {}
+    template <int G> __device__ __forceinline__ bool fine(const Step &s, unsigned) const { return isfinite(s.E); }
+};
+template <> struct Numerators<float> {
+    float top = 0.0f;
+    __device__ __forceinline__ void add(float2 n) { top = max3_abs(top, n.x, n.y); }
+    template <int G> __device__ __forceinline__ bool fine(const Step &, unsigned mask) const
+    {
+        uint32_t t = __float_as_uint(top);
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) t = max(t, __shfl_xor_sync(mask, t, o));
+        return t == 0 || (t >= __float_as_uint(QUOTIENT_MIN * 16777216.0f) && t <= __float_as_uint(QUOTIENT_MAX));
+    }
+};
+
+template <int DIM, typename T, int G, bool COMP, bool NEWTON>
 __device__ __forceinline__ Step eval_grid(const VolDesc &V, const EvolveArgs &a, const float *c, float R, int lig,
-                                          unsigned mask)
+                                          unsigned mask, Numerators<T> &numerators)
 {
     const float Ro = R + 0.5f * a.dR;
     const float Ro2 = __fmul_rn(Ro, Ro);
@@ -48,7 +91,7 @@ __device__ __forceinline__ Step eval_grid(const VolDesc &V, const EvolveArgs &a,
             const float q = __fmaf_rn(dy, dy, __fmul_rn(dz, dz));
             const float rem = __fsub_rn(Ro2, q);   // not fused: decides which voxels a chord ends on
             if (rem < 0.0f) continue;   // the row misses the ball (same for the whole group)
-            const float chord = sqrt1(fmaxf(rem, ROOT_MIN));
+            const float chord = NEWTON ? sqrt1(rem) : sqrtf(rem);
             const int i0 = (int)ceilf((c[0] - chord) * V.inv_sp[0]);
             const int i1 = (int)floorf((c[0] + chord) * V.inv_sp[0]);
             const int yy = min(max(jy, 0), V.n[1] - 1);
@@ -67,7 +110,7 @@ __device__ __forceinline__ Step eval_grid(const VolDesc &V, const EvolveArgs &a,
                                      : 0.0f;
                 const float2 d2 = fma2(dx, dx, dup2(q));
                 float2 rs;
-                const float2 r = sqrt2(make_float2(fmaxf(d2.x, ROOT_MIN), fmaxf(d2.y, ROOT_MIN)), rs);
+                const float2 r = NEWTON ? sqrt2(d2, rs) : make_float2(sqrtf(d2.x), sqrtf(d2.y));
                 const float2 t1 = fma2(r, dup2(a.inv_dr), dup2(B1)), t2 = fma2(r, dup2(a.inv_dR), dup2(B2));
                 const float2 s1 = make_float2(__saturatef(t1.x), __saturatef(t1.y));
                 const float2 s2 = make_float2(__saturatef(t2.x), __saturatef(t2.y));
@@ -79,8 +122,13 @@ __device__ __forceinline__ Step eval_grid(const VolDesc &V, const EvolveArgs &a,
                 // -S'(r) I / r, for the direction (x - c) / r (zero for a voxel on the centre)
                 const float2 k = add2(make_float2(v1 ? a.kr1 : 0.0f, w1 ? a.kr1 : 0.0f),
                                       make_float2(v2 ? a.kr2 : 0.0f, w2 ? a.kr2 : 0.0f));
-                const float2 g = div2(make_float2(__fmul_rn(d2.x > ROOT_MIN ? k.x : 0.0f, Iv),
-                                                  __fmul_rn(d2.y > ROOT_MIN ? k.y : 0.0f, Iw)), r, rs);
+                const float2 kI = make_float2(__fmul_rn(k.x, Iv), __fmul_rn(k.y, Iw));
+                float2 g;
+                if constexpr (!NEWTON)
+                    g = make_float2(d2.x > 0.0f ? kI.x / r.x : 0.0f, d2.y > 0.0f ? kI.y / r.y : 0.0f);
+                else
+                    g = div2(kI, r, rs);
+                if (NEWTON) numerators.add(kI);
                 const float gv = g.x, gw = g.y;
                 const float fv[5] = {S.x, dSdR.x, gv, gv, gv}, xv[5] = {Iv, Iv, dx.x, dy, dz};
                 const float fw[5] = {S.y, dSdR.y, gw, gw, gw}, xw[5] = {Iw, Iw, dx.y, dy, dz};
@@ -124,6 +172,16 @@ __device__ __forceinline__ Step eval_grid(const VolDesc &V, const EvolveArgs &a,
     return s;
 }
 
+// The evaluation for any operand, out of the way of the other one's registers
+template <int DIM, typename T, int G, bool COMP>
+__device__ __noinline__ Step eval_grid_any(const VolDesc &V, const EvolveArgs &a, float cx, float cy, float cz, float R,
+                                           int lig, unsigned mask)
+{
+    const float c[3] = {cx, cy, cz};
+    Numerators<T> unused;
+    return eval_grid<DIM, T, G, COMP, false>(V, a, c, R, lig, mask, unused);
+}
+
 template <int DIM, typename T, int G, bool COMP>
 __global__ void __maxnreg__(80) evolve_grid_kernel(const __grid_constant__ EvolveArgs a)
 {
@@ -142,6 +200,7 @@ __global__ void __maxnreg__(80) evolve_grid_kernel(const __grid_constant__ Evolv
         float c[3] = {V.state[k], V.state[C + k], DIM == 3 ? V.state[2 * C + k] : 0.0f};
         float R = V.state[3 * C + k];
         Step s{0.0f, 0.0f, {0.0f, 0.0f, 0.0f}};
+        bool odd = false;   // voxels that are beyond div2
         for (int n = V.first_iter; n <= V.last_iter; ++n) {
             // bounded work per evaluation: a radius beyond the grid bound (possible
             // only through an explicitly set state) stops the contour with a status
@@ -154,7 +213,14 @@ __global__ void __maxnreg__(80) evolve_grid_kernel(const __grid_constant__ Evolv
                 s.E = V.state[4 * C + k];
                 break;
             }
-            s = eval_grid<DIM, T, G, COMP>(V, a, c, R, lig, mask);
+            bool newton = !odd && newton_range(a, V, R);
+            if (newton) {
+                Numerators<T> numerators;
+                s = eval_grid<DIM, T, G, COMP, true>(V, a, c, R, lig, mask, numerators);
+                odd = !numerators.template fine<G>(s, mask);   // later balls of this contour most likely too
+                newton = !odd;
+            }
+            if (!newton) s = eval_grid_any<DIM, T, G, COMP>(V, a, c[0], c[1], c[2], R, lig, mask);
             ++evals;
             if (lig == 0) write_trace(a, v, k, n, c, R, s);
             if (!finite_step(s)) {

@@ -1,0 +1,80 @@
+"""The voxel-grid form at the ends of its range: any spacing and any voxel values that a volume
+may have.  The energy scales: with every length times a power of two (steps too) the same
+image gives the same bits, centres and radii scaled, and so does every voxel times a power
+of two (and the step size by its inverse), energies scaled; quotients at the ends of the
+range of the kernel's own division are CUDA's."""
+import dataclasses
+import math
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+def test_quotients_at_the_ends_of_their_range(tmp_path):
+    from paper_1804_06304_gb300 import build
+    exe = str(tmp_path / "quotient_range")
+    subprocess.run([build.NVCC, *build.ARCH, "-O3", "-std=c++17", "-I" + build.INCLUDE, "-o", exe,
+                    os.path.join(HERE, "_quotient_range_ref.cu")], check=True, capture_output=True)
+    assert subprocess.run([exe], check=True, capture_output=True, text=True, timeout=120).stdout.split() == ["0", "0"]
+
+
+def _evolve(ndim, dtype, s, v=1.0):
+    from paper_1804_06304_gb300 import ac
+    rng = np.random.default_rng(ndim)
+    dims = (40, 33) if ndim == 2 else (24, 20, 12)
+    image = (rng.random(dims[::-1]) * 200).astype(dtype)
+    V = ac.ac_create_volume(image * dtype(v), spacing=(s, s, 2.0 * s))
+    p = ac.default_params(ndim, 3.0, 100.0, N=1, T=6, path=ac.AC_PATH_GRID)
+    p = dataclasses.replace(p, dR=p.dR * s, Rmin=p.Rmin * s, Rmax=p.Rmax * s, max_step=p.max_step * s, eps0=p.eps0 * s * s / v)
+    C = ac.ac_seed(V, stride=4.0 * s, R0=3.0 * s)
+    ac.ac_evolve(C, p)
+    return ac.ac_get_state(C)
+
+
+# 2D energies are formed with (2R)^-2, 3D with (2R)^-3 and the voxel's volume: as far as those
+# stay normal numbers
+@pytest.mark.parametrize("ndim,exponent", [(2, -20), (2, -30), (2, -45), (2, -50), (2, 20), (2, 40), (2, 50),
+                                           (3, -20), (3, -36), (3, 20), (3, 36)])
+@pytest.mark.parametrize("dtype", [np.uint8, np.float32])
+def test_lengths_scale(ndim, dtype, exponent):
+    want, got = _evolve(ndim, dtype, 1.0), _evolve(ndim, dtype, 2.0**exponent)
+    assert np.ptp(want[3]) > 0
+    np.testing.assert_array_equal(got[:4] / np.float32(2.0**exponent), want[:4])
+    np.testing.assert_array_equal(got[4], want[4])
+
+
+@pytest.mark.parametrize("ndim", [2, 3])
+@pytest.mark.parametrize("exponent", [-95, -80, -60, 60, 80, 100])
+def test_voxels_scale(ndim, exponent):
+    want, got = _evolve(ndim, np.float32, 1.0), _evolve(ndim, np.float32, 1.0, 2.0**exponent)
+    np.testing.assert_array_equal(got[:4], want[:4])
+    np.testing.assert_array_equal(got[4] / np.float32(2.0**exponent), want[4])
+
+
+@pytest.mark.parametrize("dtype", [np.float16, np.float32])
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+def test_nonfinite_voxels_are_reported(bad, dtype):
+    """Balls with such a voxel stop with a status, those without are not touched by it."""
+    from paper_1804_06304_gb300 import ac
+    image = np.random.default_rng(1).random((40, 40)).astype(dtype)
+    seeds = np.array([[8, 8, 0, 3], [30, 30, 0, 3]], np.float32)
+    p = ac.EvolveParams(N=1, T=1, eps0=0.0, Rmin=0.5, Rmax=9.0, path=ac.AC_PATH_GRID)
+    C = ac.ac_seed(ac.ac_create_volume(image), explicit=seeds)
+    ac.ac_evolve(C, p)
+    want = ac.ac_get_state(C)
+    image[8, 8] = bad
+    C = ac.ac_seed(ac.ac_create_volume(image), explicit=seeds)
+    import torch
+    trace = torch.zeros((1, 2, 9), device="cuda")
+    ac.ac_evolve(C, p, trace=(trace, 0, 2, 1, 2))
+    with pytest.raises(ac.ACError):
+        ac.ac_get_state(C)
+    t = trace.cpu().numpy()[0]
+    assert not np.isfinite(t[0, 4]) and np.array_equal(t[1, 4:5], want[4, 1:2])
+    assert np.isfinite(t[0, 6:8]).all()   # the centre voxel has no direction
