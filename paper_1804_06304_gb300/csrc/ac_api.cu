@@ -1335,7 +1335,7 @@ __global__ void compact_active_kernel(const VolDesc *vols, int n_vols, int64_t t
 }
 
 // Device work of a prepared launch only (no host synchronisation, no allocation):
-// counters, binning by brick, sort, evolution kernel(s), kernel-time events.
+// counters, grouping by brick, evolution kernel(s), kernel-time events.
 // While a stream is captured, the kernel-time events become event-record nodes of
 // the graph (cudaEventRecordExternal), so that each replay records them.
 ac_status enqueue_prepared(Prepared &pr, Scratch &sc, cudaStream_t st, int64_t *launches, bool count = true,

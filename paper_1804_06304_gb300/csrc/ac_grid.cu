@@ -10,13 +10,13 @@
 // a row's chord, so a row is read with neighbouring addresses.  Gathers go
 // through the read-only cache from global memory.
 //
-// Bound by instruction issue (72-76 % of the slots before and after): a voxel cost 55
-// instructions, of which the square root and the division, with their paths for special
-// operands, were 22 and most of the branches; in 3D a row whose chord ends between a
-// lane's two voxels ran once for the lanes with both and once for the others.  Now the
-// two voxels of a step share packed instructions, the reciprocal root serves both root
-// and quotient, and a lane without a second voxel adds its first in the same
-// instructions.  10 iterations: 1024^2 u8 263 -> 143 us, 256x250x64 u16 1720 -> 1042 us.
+// Bound by instruction issue (1024^2 u8: 76 % of the slots; 256x250x64 u16: 81 %).  With a
+// voxel after the other, sqrtf and the division (76 and 72 %), 10 iterations took 2.11e8
+// and 1.31e9 warp instructions; in 3D a row whose chord ends between a lane's two voxels
+// ran once for the lanes with both and once for the others.  Now the two voxels of a step
+// share packed instructions, the reciprocal root serves both root and quotient, and a lane
+// without a second voxel adds its first in the same instructions: 1.17e8 and 9.61e8, the
+// kernel 263 -> 136 us and 1720 -> 1030 us.
 #include "ac_evolve.cuh"
 #include "ac_host.h"
 
