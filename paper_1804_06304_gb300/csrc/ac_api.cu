@@ -776,33 +776,34 @@ ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets
     // Every volume's bricks and, along a full brick, lattice contours: kept per axis and brick
     // size, because a launch may have many volumes and the search tries many bricks.
     const size_t n_geo = sets.size();
-    std::vector<double> counted[3];   // per size: n_geo numbers of bricks, n_geo of contours
-    std::vector<int> sizes_of[3];
-    auto along = [&](int d) -> const double * {
-        size_t k = 0;
-        while (k < sizes_of[d].size() && sizes_of[d][k] != B[d]) ++k;
-        if (k == sizes_of[d].size()) {
-            sizes_of[d].push_back(B[d]);
-            counted[d].resize(2 * n_geo * (k + 1));
-            double *t = &counted[d][2 * n_geo * k];
+    std::vector<double> counted;      // per axis and size: n_geo numbers of bricks, n_geo of contours
+    counted.reserve(2 * n_geo * 32);
+    int16_t slot[3][225] = {};        // 1 + the place of a size in `counted`
+    auto along = [&](int d) -> size_t {
+        int16_t &k = slot[d][B[d]];
+        if (k == 0) {
+            const size_t at = counted.size();
+            k = (int16_t)(1 + at / (2 * n_geo));
+            counted.resize(at + 2 * n_geo);
             for (size_t i = 0; i < n_geo; ++i) {
                 const SetGeometry &g = sets[i];
-                t[i] = d < vol->ndim ? (double)((g.n[d] + B[d] - 1) / B[d]) : 1.0;
-                t[n_geo + i] = d < vol->ndim ? std::min(lattice_along(g, d), std::ceil(B[d] * (double)g.sp[d] / stride_hint - 1e-6)) : 1.0;
+                counted[at + i] = d < vol->ndim ? (double)((g.n[d] + B[d] - 1) / B[d]) : 1.0;
+                counted[at + n_geo + i] =
+                    d < vol->ndim ? std::min(lattice_along(g, d), std::ceil(B[d] * (double)g.sp[d] / stride_hint - 1e-6)) : 1.0;
             }
         }
-        return &counted[d][2 * n_geo * k];
+        return (size_t)(k - 1) * 2 * n_geo;
     };
     auto count_bricks = [&]() {   // of the launch, for the current B
-        const double *x = along(0), *y = along(1), *z = along(2);
+        const size_t x = along(0), y = along(1), z = along(2);
         double nb = 0.0;
-        for (size_t i = 0; i < n_geo; ++i) nb += sets[i].count * x[i] * y[i] * z[i];
+        for (size_t i = 0; i < n_geo; ++i) nb += sets[i].count * counted[x + i] * counted[y + i] * counted[z + i];
         return nb;
     };
     auto full_brick = [&]() {     // the most contours that a brick holds
-        const double *x = along(0) + n_geo, *y = along(1) + n_geo, *z = along(2) + n_geo;
+        const size_t x = along(0) + n_geo, y = along(1) + n_geo, z = along(2) + n_geo;
         double full = 1.0;
-        for (size_t i = 0; i < n_geo; ++i) full = std::max(full, x[i] * y[i] * z[i]);
+        for (size_t i = 0; i < n_geo; ++i) full = std::max(full, counted[x + i] * counted[y + i] * counted[z + i]);
         return full;
     };
     for (int d = 0; d < vol->ndim; ++d) B[d] = brick_of(d);
