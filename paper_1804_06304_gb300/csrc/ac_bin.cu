@@ -244,10 +244,14 @@ __device__ __forceinline__ void order_list(uint32_t *list, uint32_t *tmp, uint32
 }
 
 // A block looks at 32 bricks, gridDim.x apart, in one load.  `tmp` holds a word per contour.
+// Most launches have nothing to order: the kernel is launched while the scatter still runs
+// (programmatic dependent launch) and waits for it here, so that it costs them nothing
+// (after the scatter: 4 us, 145 -> 149 us for 900x800 u16).
 __global__ void __launch_bounds__(ORDER_THREADS) bin_order_kernel(const uint2 *ranges, int64_t nb, const uint32_t *head,
                                                                   uint32_t *order, uint32_t *tmp)
 {
     __shared__ uint32_t words[WORDS], warp_sums[32];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (head[1] == 0) return;
     for (int64_t b = blockIdx.x; b < nb; b += 32 * (int64_t)gridDim.x) {
         const int64_t mine = b + (int64_t)(threadIdx.x & 31) * gridDim.x;
@@ -349,9 +353,21 @@ cudaError_t launch_bin(const EvolveArgs &a, const BinSpace &s, cudaStream_t st, 
                                                       a.path_counts);
     bin_alloc_kernel<<<blocks_of(bricks), 256, 0, st>>>(ranges, bricks, static_cast<uint32_t *>(s.table));
     bin_scatter_kernel<<<blocks_of(total), 256, 0, st>>>(ranges, s.keys, s.ranks, total, s.order);
-    // the keys have been read: their space serves the ordering
-    bin_order_kernel<<<(unsigned)std::min<int64_t>(bricks, 304), ORDER_THREADS, 0, st>>>(
-        ranges, bricks, static_cast<const uint32_t *>(s.table), s.order, s.keys);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    // the keys have been read when it starts to order: their space serves it
+    cudaLaunchConfig_t order{};
+    order.gridDim = dim3((unsigned)std::min<int64_t>(bricks, 152));
+    order.blockDim = dim3(ORDER_THREADS);
+    order.stream = st;
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    order.attrs = &early;
+    order.numAttrs = 1;
+    e = cudaLaunchKernelEx(&order, bin_order_kernel, (const uint2 *)ranges, bricks, static_cast<const uint32_t *>(s.table),
+                           s.order, s.keys);
+    if (e != cudaSuccess) return e;
     *launches += 4;
     return cudaGetLastError();
 }

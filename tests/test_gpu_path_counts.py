@@ -55,3 +55,21 @@ def test_crowded_bricks_are_sorted(n, launches):
     before = ac.ac_kernel_launches()
     ac.ac_evolve(C, ac.EvolveParams(N=64, T=1, eps0=0.0, Rmin=0.5, Rmax=1.5, brick=(8, 8, 0)))
     assert ac.ac_kernel_launches() - before == launches
+
+
+@pytest.mark.parametrize("n", [5000, 20000])
+def test_counts_of_a_replayed_graph(n):
+    """The grouping as part of a captured graph (its last kernel is launched ahead of the end of the
+    one before): every replay counts what a plain launch counts."""
+    from paper_1804_06304_gb300 import ac
+    rng = np.random.default_rng(n)
+    V = ac.ac_create_volume(rng.integers(0, 255, size=(256, 256), dtype=np.uint8))
+    seeds = np.column_stack([rng.uniform(0, 40, (n, 2)), np.zeros(n), rng.uniform(0.6, 1.0, n)]).astype(np.float32)
+    p = ac.EvolveParams(N=64, T=2, eps0=0.0, Rmin=0.5, Rmax=1.5, seed=5, brick=(8, 8, 0), halo_factor=1.0)
+    C = ac.ac_seed(V, explicit=seeds)
+    ac.ac_evolve(C, p)
+    want = ac.ac_evolve_stats(C)
+    plan = ac.ac_plan_create([C], p)
+    for _ in range(4):
+        ac.ac_plan_launch(plan, use_graph=True)
+        assert ac.ac_evolve_stats(C) == want
