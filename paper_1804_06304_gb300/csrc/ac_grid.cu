@@ -16,7 +16,7 @@
 // ran once for the lanes with both and once for the others.  Now the two voxels of a step
 // share packed instructions, the reciprocal root serves both root and quotient, and a lane
 // without a second voxel adds its first in the same instructions: 1.17e8 and 9.61e8, the
-// kernel 263 -> 136 us and 1720 -> 1030 us.
+// kernel 263 -> 133 us and 1720 -> 1022 us.
 #include "ac_evolve.cuh"
 #include "ac_host.h"
 
@@ -172,14 +172,39 @@ __device__ __forceinline__ Step eval_grid(const VolDesc &V, const EvolveArgs &a,
     return s;
 }
 
-// The evaluation for any operand, out of the way of the other one's registers
-template <int DIM, typename T, int G, bool COMP>
-__device__ __noinline__ Step eval_grid_any(const VolDesc &V, const EvolveArgs &a, float cx, float cy, float cz, float R,
-                                           int lig, unsigned mask)
+// Iterations n, n + 1, ... of a contour in registers, to the last of its window or until it
+// stops (returns last_iter + 1), or (NEWTON) until one that is beyond the Newton steps
+// (returns its number, nothing done).
+template <int DIM, typename T, int G, bool COMP, bool NEWTON>
+__device__ __forceinline__ int run_grid(const VolDesc &V, const EvolveArgs &a, int v, int64_t k, int n, int lig, unsigned mask,
+                                        float *c, float &R, int32_t &h, Step &s, unsigned int &evals)
 {
-    const float c[3] = {cx, cy, cz};
-    Numerators<T> unused;
-    return eval_grid<DIM, T, G, COMP, false>(V, a, c, R, lig, mask, unused);
+    for (; n <= V.last_iter; ++n) {
+        // bounded work per evaluation: a radius beyond the grid bound (possible
+        // only through an explicitly set state) stops the contour with a status
+        const float Ro = R + 0.5f * a.dR;
+        bool wide = false;
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) wide = wide || !(Ro * V.inv_sp[d] <= GRID_MAX_RADIUS_VOXELS);
+        if (wide) {
+            if (lig == 0) atomicOr(V.status, STATUS_GRID_RANGE);
+            s.E = V.state[4 * V.C + k];
+            break;
+        }
+        if (NEWTON && !newton_range(a, V, R)) return n;
+        Numerators<T> numerators;
+        const Step t = eval_grid<DIM, T, G, COMP, NEWTON>(V, a, c, R, lig, mask, numerators);
+        if (NEWTON && !numerators.template fine<G>(t, mask)) return n;
+        s = t;
+        ++evals;
+        if (lig == 0) write_trace(a, v, k, n, c, R, s);
+        if (!finite_step(s)) {
+            if (lig == 0) atomicOr(V.status, STATUS_NONFINITE);
+            break;
+        }
+        if (step_or_stop<DIM>(s, n, a, V, c, R, h)) break;
+    }
+    return V.last_iter + 1;
 }
 
 template <int DIM, typename T, int G, bool COMP>
@@ -200,35 +225,9 @@ __global__ void __maxnreg__(80) evolve_grid_kernel(const __grid_constant__ Evolv
         float c[3] = {V.state[k], V.state[C + k], DIM == 3 ? V.state[2 * C + k] : 0.0f};
         float R = V.state[3 * C + k];
         Step s{0.0f, 0.0f, {0.0f, 0.0f, 0.0f}};
-        bool odd = false;   // voxels that are beyond div2
-        for (int n = V.first_iter; n <= V.last_iter; ++n) {
-            // bounded work per evaluation: a radius beyond the grid bound (possible
-            // only through an explicitly set state) stops the contour with a status
-            const float Ro = R + 0.5f * a.dR;
-            bool wide = false;
-#pragma unroll
-            for (int d = 0; d < DIM; ++d) wide = wide || !(Ro * V.inv_sp[d] <= GRID_MAX_RADIUS_VOXELS);
-            if (wide) {
-                if (lig == 0) atomicOr(V.status, STATUS_GRID_RANGE);
-                s.E = V.state[4 * C + k];
-                break;
-            }
-            bool newton = !odd && newton_range(a, V, R);
-            if (newton) {
-                Numerators<T> numerators;
-                s = eval_grid<DIM, T, G, COMP, true>(V, a, c, R, lig, mask, numerators);
-                odd = !numerators.template fine<G>(s, mask);   // later balls of this contour most likely too
-                newton = !odd;
-            }
-            if (!newton) s = eval_grid_any<DIM, T, G, COMP>(V, a, c[0], c[1], c[2], R, lig, mask);
-            ++evals;
-            if (lig == 0) write_trace(a, v, k, n, c, R, s);
-            if (!finite_step(s)) {
-                if (lig == 0) atomicOr(V.status, STATUS_NONFINITE);
-                break;
-            }
-            if (step_or_stop<DIM>(s, n, a, V, c, R, h)) break;
-        }
+        const int n = run_grid<DIM, T, G, COMP, true>(V, a, v, k, V.first_iter, lig, mask, c, R, h, s, evals);
+        if (n <= V.last_iter)   // the rest of its window in the general form
+            run_grid<DIM, T, G, COMP, false>(V, a, v, k, n, lig, mask, c, R, h, s, evals);
         if (lig == 0) {
             V.state[k] = c[0];
             V.state[C + k] = c[1];
