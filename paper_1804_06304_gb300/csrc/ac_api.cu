@@ -341,6 +341,39 @@ static ac_status make_contours(ac_volume *vol, int64_t C, ac_contours **out, cud
 static ac_status seed_impl(ac_volume *vol, const ac_seed_params *params, const float *explicit_cR,
                            int64_t n_explicit, void *cuda_stream, ac_contours **out, cudaMemPool_t pool);
 
+// Explicit seeds need not cover their volume.  Seeds crowded in a part of it (CROWD and more
+// for each lattice cell that holds any) are planned for as such, in volumes small enough
+// that their bricks are chosen by an estimate: taken for a lattice, 3,000 seeds in a corner
+// of 128^3 took 7.4 ms (3.5 ms before there was an estimate; 0.58 ms with it knowing).
+// Below CROWD a lattice's layouts are as good or better (160x160x80, 2.5 per cell: 581 us
+// against 660).
+static void find_crowding(ac_contours *c, const float *soa)
+{
+    constexpr double CROWD = 3.0;
+    const ac_volume *v = c->vol;
+    int64_t L[3] = {1, 1, 1}, cells = 1;
+    for (int d = 0; d < v->ndim; ++d) {
+        const double along = std::floor(v->n[d] * (double)v->sp[d] / c->stride_hint);
+        L[d] = (int64_t)std::max(1.0, std::min(along, (double)(1 << 20)));
+        cells = std::min(cells * L[d], (int64_t)1 << 40);
+    }
+    if (cells > 1 << 20 || c->C < 2 * CROWD) return;
+    std::vector<bool> held((size_t)cells);
+    int64_t occupied = 0;
+    for (int64_t k = 0; k < c->C; ++k) {
+        int64_t at = 0;
+        for (int d = v->ndim - 1; d >= 0; --d) {
+            const double x = (soa[(size_t)(d * c->C + k)] / v->sp[d] + 0.5) / v->n[d] * L[d];
+            at = at * L[d] + std::max<int64_t>(0, std::min(L[d] - 1, (int64_t)x));
+        }
+        occupied += held[(size_t)at] ? 0 : 1;
+        held[(size_t)at] = true;
+    }
+    if (c->C < CROWD * occupied) return;
+    c->density = (double)c->C / occupied;
+    c->filled = (double)occupied / cells;
+}
+
 extern "C" ac_status ac_seed(ac_volume *vol, const ac_seed_params *params, const float *explicit_cR,
                              int64_t n_explicit, void *cuda_stream, ac_contours **out)
 {
@@ -397,6 +430,7 @@ static ac_status seed_impl(ac_volume *vol, const ac_seed_params *params, const f
         }
         c->r_hint = rmax;
         c->stride_hint = std::sqrt(1.5) * rmax;
+        find_crowding(c, soa.data());
         *out = c;
         return AC_OK;
     }
@@ -665,10 +699,12 @@ ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets
         if (G == 16) cells[1] = 4;
         if (G == 8 && p->N >= 512) cells[0] = cells[1] = cells[2] = 4;
     }
-    // groups for the contours of a brick (lattice estimate), 1..16 warps
+    // groups for the contours of a brick (lattice estimate, more of them where the bricks of a
+    // crowded set are chosen by estimate), 1..16 warps
+    double crowding = 1.0;
     auto warps_of = [&]() {
         if (p->warps_per_block) return p->warps_per_block;
-        double per = 1.0;
+        double per = crowding;
         for (int d = 0; d < vol->ndim; ++d) per *= std::max(1.0, B[d] * (double)vol->sp[d] / stride_hint);
         return std::max(1, std::min(16, (int)std::ceil(per * G / 32.0)));
     };
@@ -800,10 +836,21 @@ ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets
         for (size_t i = 0; i < n_geo; ++i) nb += sets[i].count * counted[x + i] * counted[y + i] * counted[z + i];
         return nb;
     };
+    auto active_bricks = [&]() {  // those with contours, if a set's occupied cells lie anywhere
+        const size_t x = along(0), y = along(1), z = along(2);
+        double nb = 0.0;
+        for (size_t i = 0; i < n_geo; ++i) {
+            double one = sets[i].count * counted[x + i] * counted[y + i] * counted[z + i];
+            if (sets[i].filled < 1.0)
+                one *= 1.0 - std::pow(1.0 - sets[i].filled, counted[x + n_geo + i] * counted[y + n_geo + i] * counted[z + n_geo + i]);
+            nb += one;
+        }
+        return nb;
+    };
     auto full_brick = [&]() {     // the most contours that a brick holds
         const size_t x = along(0) + n_geo, y = along(1) + n_geo, z = along(2) + n_geo;
         double full = 1.0;
-        for (size_t i = 0; i < n_geo; ++i) full = std::max(full, counted[x + i] * counted[y + i] * counted[z + i]);
+        for (size_t i = 0; i < n_geo; ++i) full = std::max(full, std::ceil(sets[i].density * counted[x + i] * counted[y + i] * counted[z + i]));
         return full;
     };
     for (int d = 0; d < vol->ndim; ++d) B[d] = brick_of(d);
@@ -830,11 +877,12 @@ ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets
             small = small || nb < 1216;
         }
         if (small) {
-            double lattice = 0.0;
+            double contours = 0.0;
             for (const SetGeometry &g : sets) {
-                double one = (double)g.count;
+                double one = g.count * (g.density * g.filled);
                 for (int d = 0; d < vol->ndim; ++d) one *= lattice_along(g, d);
-                lattice += one;
+                contours += one;
+                crowding = std::max(crowding, g.density);
             }
             const int reg_warps = vol->ndim == 3 ? 16 : 21;   // warps an SM's registers hold
             const double per_warp = 32.0 / G;                 // contours a warp evolves at once
@@ -859,9 +907,9 @@ ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets
                 return 32.0 * sq / (sum * sum);
             };
             auto estimate = [&](int warps, int smem) {
-                const double nb = count_bricks(), full = full_brick();
+                const double nb = active_bricks(), full = full_brick();
                 const int r = std::max(1, std::min({reg_warps / warps, SM_SMEM / (smem + BRICK_SMEM_EXTRA), 32}));
-                const double busy = std::min(lattice / nb / per_warp, (double)warps);   // warps at work, on average
+                const double busy = std::min(contours / nb / per_warp, (double)warps);   // warps at work, on average
                 const double most = std::min((double)warps, std::ceil(full / per_warp));
                 const double passes = std::ceil(full / per_warp / warps);
                 const double quads = vol->ndim == 2 && vol->dtype != AC_F32 ? smem / (8.0 + vol->es) / (warps * 32) * 1000.0 : 0.0;
@@ -936,6 +984,8 @@ void launch_geometry(ac_contours *const *sets, int n_sets, double stride_hint, a
         SetGeometry g;
         std::memset(&g, 0, sizeof(g));
         g.count = 1;
+        g.density = sets[i]->density;
+        g.filled = sets[i]->filled;
         double lattice = 1.0;
         for (int d = 0; d < 3; ++d) {
             g.n[d] = v->n[d];
@@ -948,7 +998,8 @@ void launch_geometry(ac_contours *const *sets, int n_sets, double stride_hint, a
             for (int d = 0; d < 3; ++d) vol.sp[d] = g.sp[d];
         }
         if (!all.empty() && std::memcmp(all.back().n, g.n, sizeof(g.n)) == 0 &&
-            std::memcmp(all.back().sp, g.sp, sizeof(g.sp)) == 0)
+            std::memcmp(all.back().sp, g.sp, sizeof(g.sp)) == 0 && all.back().density == g.density &&
+            all.back().filled == g.filled)
             ++all.back().count;
         else
             all.push_back(g);
@@ -964,6 +1015,7 @@ std::vector<SetGeometry> one_volume(const ac_volume &v)
         g.sp[d] = v.sp[d];
     }
     g.count = 1;
+    g.density = g.filled = 1.0;
     return {g};
 }
 

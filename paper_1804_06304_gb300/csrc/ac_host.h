@@ -97,11 +97,13 @@ struct PlanKey {
     float sp[3], dR, halo_factor;
     int dtype, ndim, N, T, path, lanes, comp, warps, sampling, brick[3];
 };
-// Volumes of one geometry among a launch's sets
+// Volumes of one geometry (and crowding) among a launch's sets
 struct SetGeometry {
     int64_t n[3];
-    float sp[3];
+    double density, filled;   // see ac_contours
     int64_t count;
+    float sp[3];
+    int32_t pad;              // compared byte by byte
 };
 struct PlanMemo {
     bool valid = false;
@@ -130,6 +132,9 @@ struct ac_contours {
     unsigned long long *path_counts = nullptr;   // device [3]: contour-iterations per gather path
     double stride_hint = 0;   // lattice stride (or mean spacing of explicit seeds)
     double r_hint = 0;        // largest initial radius
+    // Crowded explicit seeds: contours per lattice cell that holds any, and the share of cells
+    // that do (1 and 1: like a lattice)
+    double density = 1, filled = 1;
     ac::Scratch scratch;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;  // around the last evolution kernel(s)
     bool lattice = false;                       // lattice-seeded: parameters below
