@@ -270,6 +270,7 @@ __global__ void cell_scatter_kernel(int64_t n, const uint32_t *cell, uint32_t *r
 // contours: set after set 2,105 us, in turn 401 us; of 1,000 sets of 500 398 and 101 us.
 constexpr int LOOKS = 64;
 constexpr int ROUND_WARPS = 8;
+constexpr int64_t RESIDENT_WARPS = 152 * 64;
 constexpr uint32_t NONE = 0xffffffffu;
 
 __global__ void __launch_bounds__(32 * ROUND_WARPS) round_kernel(const LocSet *sets, int nsets, const float4 *pos, int64_t n,
@@ -635,9 +636,10 @@ ac_status localize_many(ac_contours *const *sets, const float *E0, ac_cell *cons
     LC_CUDA(sc.cub.ensure(tmp));
     const int64_t max_rounds = localize_round_limit(n_max);
     // blocks of the sets' heads: the largest set whole if at most three in four blocks then
-    // have nothing to do
+    // have nothing to do; none where the GPU holds nearly all survivors at once anyway (8 sets
+    // of 2,000 among 40: 40 us set after set, 50 us in turn)
     const int64_t in_order = (n + ROUND_WARPS - 1) / ROUND_WARPS, largest = (n_max + ROUND_WARPS - 1) / ROUND_WARPS;
-    const int64_t heads = nsets > 1 ? std::min(largest, 4 * in_order / nsets) : 0;
+    const int64_t heads = nsets > 1 && n > 2 * RESIDENT_WARPS ? std::min(largest, 4 * in_order / nsets) : 0;
     const unsigned round_blocks = (unsigned)(heads * nsets + (heads < largest ? in_order : 0));
     const bool few = n <= 16384;   // 400 KB of cells: less than another synchronisation costs
     int64_t rounds = 0;
