@@ -16,7 +16,8 @@
 // per brick, passes of 10 iterations went from 111 to 99 us (64x64x32, 2,048 contours),
 // 226 to 189 us (512^2), 547 to 504 us (128^3), 2.07 to 2.00 ms (4096^2) and 53.8 to
 // 52.7 ms (1024x1024x256, where a CTA has its SM alone while it searches).  Where bricks
-// far outnumber contours (see bin_by_sort) the contours are still sorted by brick.
+// far outnumber contours, or hold hundreds each (see bin_by_sort), the contours are still
+// sorted by brick.
 #include <cub/cub.cuh>
 
 #include "ac_host.h"

@@ -10,12 +10,12 @@
 // a row's chord, so a row is read with neighbouring addresses.  Gathers go
 // through the read-only cache from global memory.
 //
-// Bound by instruction issue (1024^2 u8: 76 % of the slots; 256x250x64 u16: 81 %).  With a
+// Bound by instruction issue (1024^2 u8: 76 % of the slots; 256x250x64 u16: 80 %).  With a
 // voxel after the other, sqrtf and the division (76 and 72 %), 10 iterations took 2.11e8
 // and 1.31e9 warp instructions; in 3D a row whose chord ends between a lane's two voxels
 // ran once for the lanes with both and once for the others.  Now the two voxels of a step
 // share packed instructions, the reciprocal root serves both root and quotient, and a lane
-// without a second voxel adds its first in the same instructions: 1.17e8 and 9.61e8, the
+// without a second voxel adds its first in the same instructions: 1.14e8 and 9.47e8, the
 // kernel 263 -> 133 us and 1720 -> 1022 us.
 #include "ac_evolve.cuh"
 #include "ac_host.h"
