@@ -972,8 +972,9 @@ ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets
 // longest of them, with the spacing of the volume with the most lattice contours, whatever
 // the order of the sets.  Planned for the first volume alone, a launch over 30 volumes of
 // 128^3 behind one of 40x40x20 took 74.9 ms (that volume's bricks and regions), in the
-// opposite order 7.4 ms.
-void launch_geometry(ac_contours *const *sets, int n_sets, double stride_hint, ac_volume &vol,
+// opposite order 7.4 ms.  Bricks that the caller gives are cut to the first volume, and their
+// regions with them: what fits there must go on fitting.
+void launch_geometry(ac_contours *const *sets, int n_sets, double stride_hint, bool own_bricks, ac_volume &vol,
                      std::vector<SetGeometry> &all)
 {
     vol = *sets[0]->vol;   // voxel type and dimensions are common
@@ -990,12 +991,12 @@ void launch_geometry(ac_contours *const *sets, int n_sets, double stride_hint, a
         for (int d = 0; d < 3; ++d) {
             g.n[d] = v->n[d];
             g.sp[d] = v->sp[d];
-            vol.n[d] = std::max(vol.n[d], v->n[d]);
+            if (own_bricks) vol.n[d] = std::max(vol.n[d], v->n[d]);
             if (d < v->ndim) lattice *= std::max(1.0, std::floor(v->n[d] * (double)v->sp[d] / stride_hint));
         }
         if (lattice > most || (lattice == most && std::lexicographical_compare(vol.sp, vol.sp + 3, g.sp, g.sp + 3))) {
             most = lattice;
-            for (int d = 0; d < 3; ++d) vol.sp[d] = g.sp[d];
+            for (int d = 0; d < 3 && own_bricks; ++d) vol.sp[d] = g.sp[d];
         }
         if (!all.empty() && std::memcmp(all.back().n, g.n, sizeof(g.n)) == 0 &&
             std::memcmp(all.back().sp, g.sp, sizeof(g.sp)) == 0 && all.back().density == g.density &&
@@ -1220,7 +1221,7 @@ ac_status prepare_sets(ac_contours *const *sets, const ac_batch_item *items, int
     Plan &pl = pr.pl;
     ac_volume common;
     std::vector<SetGeometry> geometry;
-    launch_geometry(sets, n_sets, stride_hint, common, geometry);
+    launch_geometry(sets, n_sets, stride_hint, !p->brick[0] && !p->brick[1] && !p->brick[2], common, geometry);
     s = plan_with_memo(&common, std::move(geometry), stride_hint, r_hint, p, sc.memo, pl);
     if (s != AC_OK) return s;
     pr.dtype = v0->dtype;

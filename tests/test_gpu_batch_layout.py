@@ -31,3 +31,21 @@ def test_order_of_the_sets_does_not_matter(ndim, dims, spacings, N):
         assert c == counts[0]
         for i in s:
             np.testing.assert_array_equal(s[i], states[0][i])
+
+
+def test_bricks_of_the_callers_fit_a_small_first_volume():
+    """Bricks too large for a staged region are cut to the first volume: such a batch is taken as
+    long as that one is small, and gives what every set gives alone."""
+    from paper_1804_06304_gb300 import ac
+    rng = np.random.default_rng(3)
+    dims = [(20, 12, 9), (60, 60, 60), (44, 50, 41)]
+    p = ac.EvolveParams(N=33, T=4, eps0=0.02, Rmin=0.5, Rmax=6.0, seed=5, brick=(60, 60, 60))
+    volumes = [ac.ac_create_volume(rng.random(d[::-1]).astype(np.float32)) for d in dims]
+    sets = [ac.ac_seed(v, stride=5.0) for v in volumes]
+    ac.ac_evolve_batch(sets, p)
+    for c, v in zip(sets, volumes):
+        alone = ac.ac_seed(v, stride=5.0)
+        ac.ac_evolve(alone, ac.EvolveParams(N=33, T=4, eps0=0.02, Rmin=0.5, Rmax=6.0, seed=5))
+        np.testing.assert_array_equal(ac.ac_get_state(c), ac.ac_get_state(alone))
+    with pytest.raises(ac.ACError):
+        ac.ac_evolve_batch(sets[::-1], p)
