@@ -26,17 +26,17 @@ namespace {
 // Whether the roots and quotients of an evaluation with radius R are Newton steps.  Voxels
 // nearer to the centre than the root of ROOT_MIN have a root that is only near enough: they
 // must lie inside both bands, where the root plays no part.  Squared distances, also of the
-// voxel beside a chord's last, and (integer voxels) k I stay within the ranges of sqrt2 and
-// div2.  What remains (spacings below about 1e-14 or above 1e7, radii below half a band)
-// takes the operations for any operand; there a chord of ROOT_MIN's root would be
-// thousands of voxels long.
-__device__ __forceinline__ bool newton_range(const EvolveArgs &a, const VolDesc &V, float R)
+// voxel beside a chord's last, squared half chords (zero, or at least 2^-48 of the squared
+// radius in 2D, where the difference is fused, 2^-25 in 3D) and (integer voxels) k I stay
+// within the ranges of sqrt2 and div2.  What remains (radii below 1e-7 in 2D and 3e-11 in 3D,
+// spacings above 3e7, radii of half a band and less) takes the operations for any operand.
+template <int DIM> __device__ __forceinline__ bool newton_range(const EvolveArgs &a, const VolDesc &V, float R)
 {
     constexpr float NEAR = 7.105427357601002e-15f;   // 2^-47
     const float Ro = R + 0.5f * a.dR, Ro2 = __fmul_rn(Ro, Ro);
     const float kmin = fminf(fabsf(a.kr1), fabsf(a.kr2)), kmax = fmaxf(fabsf(a.kr1), fabsf(a.kr2));
-    return Ro2 > 8.470329472543003e-22f && Ro2 < 1.125899906842624e15f &&   // 2^-70, 2^50
-           V.sp[0] < 33554432.0f &&                                         // 2^25
+    return Ro2 > (DIM == 2 ? 1.4210854715202004e-14f : 8.470329472543003e-22f) &&   // 2^-46, 2^-70
+           Ro2 < 1.125899906842624e15f && V.sp[0] < 33554432.0f &&                  // 2^50, 2^25
            fmaf(-a.rho * R + NEAR, a.inv_dr, 0.5f) < -0.001f && fmaf(NEAR - R, a.inv_dR, 0.5f) < -0.001f &&
            kmin > 9.094947017729282e-13f && kmax < 1.099511627776e12f;      // 2^-40, 2^40
 }
@@ -89,7 +89,8 @@ __device__ __forceinline__ Step eval_grid(const VolDesc &V, const EvolveArgs &a,
         for (int jy = lo[1]; jy <= hi[1]; ++jy) {
             const float dy = fmaf((float)jy, V.sp[1], -c[1]);
             const float q = __fmaf_rn(dy, dy, __fmul_rn(dz, dz));
-            const float rem = __fsub_rn(Ro2, q);   // not fused: decides which voxels a chord ends on
+            // fused in 2D, not in 3D: decides which voxels a chord ends on
+            const float rem = DIM == 2 ? __fmaf_rn(Ro, Ro, -q) : __fsub_rn(Ro2, q);
             if (rem < 0.0f) continue;   // the row misses the ball (same for the whole group)
             const float chord = NEWTON ? sqrt1(rem) : sqrtf(rem);
             const int i0 = (int)ceilf((c[0] - chord) * V.inv_sp[0]);
@@ -191,7 +192,7 @@ __device__ __forceinline__ int run_grid(const VolDesc &V, const EvolveArgs &a, i
             s.E = V.state[4 * V.C + k];
             break;
         }
-        if (NEWTON && !newton_range(a, V, R)) return n;
+        if (NEWTON && !newton_range<DIM>(a, V, R)) return n;
         Numerators<T> numerators;
         const Step t = eval_grid<DIM, T, G, COMP, NEWTON>(V, a, c, R, lig, mask, numerators);
         if (NEWTON && !numerators.template fine<G>(t, mask)) return n;

@@ -78,3 +78,46 @@ def test_nonfinite_voxels_are_reported(bad, dtype):
     t = trace.cpu().numpy()[0]
     assert not np.isfinite(t[0, 4]) and np.array_equal(t[1, 4:5], want[4, 1:2])
     assert np.isfinite(t[0, 6:8]).all()   # the centre voxel has no direction
+
+
+# balls with a voxel within half a unit in the last place of their border: the rows in which it lies
+# end with or without it, by whether Ro^2 - dy^2 is rounded once or twice
+BORDER = [(1.7738727, 5.1184683, 10.407612), (4.389767, 4.105155, 11.386679), (6.4855967, 2.9813597, 9.075569),
+          (7.028953, 5.40722, 11.078195), (0.670507, 4.689889, 11.703898), (0.19110374, 5.8286586, 8.98151),
+          (0.95753396, 1.2068299, 8.581024), (0.53011334, 1.3633039, 10.179406), (7.610154, 3.7508016, 11.948878),
+          (1.1282305, 2.1320808, 11.602594), (0.6849803, 2.5642705, 11.291962)]
+
+
+@pytest.mark.parametrize("lanes", [0, 8, 16])
+def test_rows_end_where_the_fused_difference_says(lanes):
+    """A ball's dE/dR over a constant image, in 64 bits over the voxels of the rows that binary32 gives
+    with Ro^2 - dy^2 rounded once; a voxel more or less changes it by 2e-2 and more, rounding by 1e-4."""
+    import torch
+    from paper_1804_06304_gb300 import ac
+    f = np.float32
+    sp = np.array([0.5, 0.7], f)
+    V = ac.ac_create_volume(np.full((10, 18), 100, np.uint8), spacing=(0.5, 0.7, 1.0))
+    seeds = np.array([(x, y, 0.0, r) for x, y, r in BORDER], f)
+    C = ac.ac_seed(V, explicit=seeds)
+    trace = torch.zeros((1, len(seeds), 9), device="cuda")
+    p = ac.EvolveParams(N=64, T=1, eps0=0.0, Rmin=0.5, Rmax=22.0, path=ac.AC_PATH_GRID, lanes_per_contour=lanes)
+    ac.ac_evolve(C, p, trace=(trace, 0, len(seeds), 1, 2))
+    inv, rho = f(1) / sp, 2.0 ** -0.5
+    for t, (x, y, _, R) in zip(trace.cpu().numpy()[0], seeds):
+        Ro = f(R + f(0.5))
+        sums = np.zeros(2)
+        for j in range(int(np.ceil(f(f(y - Ro) * inv[1]))), int(np.floor(f(f(y + Ro) * inv[1]))) + 1):
+            dy = f(float(f(j)) * float(sp[1]) - float(y))
+            rem = f(float(Ro) ** 2 - float(f(dy * dy)))   # exact in 64 bits, rounded once
+            if rem < 0:
+                continue
+            chord = np.sqrt(rem)
+            i = np.arange(int(np.ceil(f(f(x - chord) * inv[0]))), int(np.floor(f(f(x + chord) * inv[0]))) + 1)
+            r = np.hypot(i * float(sp[0]) - float(x), float(dy))
+            t1, t2 = (r - rho * float(R)) / rho + 0.5, r - float(R) + 0.5
+            border = np.abs(t2 - 1.0) < 1e-6    # in the band: a voxel of the ball
+            t2 = np.where(border, 1.0, t2)
+            sums[0] += (-1.0 + 2.0 * np.clip(t1, 0, 1) - np.clip(t2, 0, 1)).sum()
+            sums[1] += (-2.0 * ((t1 >= 0) & (t1 <= 1)) + ((t2 >= 0) & (t2 <= 1))).sum()
+        want = (sums[1] - 2.0 * sums[0] / float(R)) * 100.0 * 0.5 * 0.7 / (2.0 * float(R)) ** 2
+        assert abs(float(t[5]) - want) < 1e-2, (x, y, R, t[5], want)
