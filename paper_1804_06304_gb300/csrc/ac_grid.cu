@@ -23,22 +23,39 @@
 namespace ac {
 namespace {
 
-// Whether the roots and quotients of an evaluation with radius R are Newton steps.  Voxels
-// nearer to the centre than the root of ROOT_MIN have a root that is only near enough: they
-// must lie inside both bands, where the root plays no part.  Squared distances, also of the
+// Whether the voxel nearest to c lies off it, but nearer than the root of ROOT_MIN (a little
+// more, for rounding)
+template <int DIM> __device__ __forceinline__ bool near_centre(const VolDesc &V, const float *c)
+{
+    float d2 = 0.0f, least = 0.0f;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+        const float off = fabsf(fmaf(rintf(c[d] * V.inv_sp[d]), V.sp[d], -c[d]));
+        d2 = fmaf(off, off, d2);
+        least = fmaxf(least, off);
+    }
+    return least > 0.0f && d2 < 4.0f * ROOT_MIN;
+}
+
+// Whether the roots and quotients of an evaluation with centre c and radius R are Newton
+// steps.  Voxels nearer to the centre than the root of ROOT_MIN (but not on it) have a root that
+// is only near enough: they must lie inside both bands, where the root plays no part, or not
+// be there (none but the nearest can).  Squared distances, also of the
 // voxel beside a chord's last, squared half chords (zero, or at least 2^-48 of the squared
 // radius in 2D, where the difference is fused, 2^-25 in 3D) and (integer voxels) k I stay
 // within the ranges of sqrt2 and div2.  What remains (radii below 1e-7 in 2D and 3e-11 in 3D,
-// spacings above 3e7, radii of half a band and less) takes the operations for any operand.
-template <int DIM> __device__ __forceinline__ bool newton_range(const EvolveArgs &a, const VolDesc &V, float R)
+// spacings above 3e7) takes the operations for any operand.
+template <int DIM>
+__device__ __forceinline__ bool newton_range(const EvolveArgs &a, const VolDesc &V, const float *c, float R)
 {
     constexpr float NEAR = 7.105427357601002e-15f;   // 2^-47
     const float Ro = R + 0.5f * a.dR, Ro2 = __fmul_rn(Ro, Ro);
     const float kmin = fminf(fabsf(a.kr1), fabsf(a.kr2)), kmax = fmaxf(fabsf(a.kr1), fabsf(a.kr2));
     return Ro2 > (DIM == 2 ? 1.4210854715202004e-14f : 8.470329472543003e-22f) &&   // 2^-46, 2^-70
            Ro2 < 1.125899906842624e15f && V.sp[0] < 33554432.0f &&                  // 2^50, 2^25
-           fmaf(-a.rho * R + NEAR, a.inv_dr, 0.5f) < -0.001f && fmaf(NEAR - R, a.inv_dR, 0.5f) < -0.001f &&
-           kmin > 9.094947017729282e-13f && kmax < 1.099511627776e12f;      // 2^-40, 2^40
+           kmin > 9.094947017729282e-13f && kmax < 1.099511627776e12f &&            // 2^-40, 2^40
+           ((fmaf(-a.rho * R + NEAR, a.inv_dr, 0.5f) < -0.001f && fmaf(NEAR - R, a.inv_dR, 0.5f) < -0.001f) ||
+            !near_centre<DIM>(V, c));
 }
 
 // Whether div2 was right for all numerators of a ball, known after it (`s`: the evaluation).
@@ -192,7 +209,7 @@ __device__ __forceinline__ int run_grid(const VolDesc &V, const EvolveArgs &a, i
             s.E = V.state[4 * V.C + k];
             break;
         }
-        if (NEWTON && !newton_range<DIM>(a, V, R)) return n;
+        if (NEWTON && !newton_range<DIM>(a, V, c, R)) return n;
         Numerators<T> numerators;
         const Step t = eval_grid<DIM, T, G, COMP, NEWTON>(V, a, c, R, lig, mask, numerators);
         if (NEWTON && !numerators.template fine<G>(t, mask)) return n;

@@ -121,3 +121,42 @@ def test_rows_end_where_the_fused_difference_says(lanes):
             sums[1] += (-2.0 * ((t1 >= 0) & (t1 <= 1)) + ((t2 >= 0) & (t2 <= 1))).sum()
         want = (sums[1] - 2.0 * sums[0] / float(R)) * 100.0 * 0.5 * 0.7 / (2.0 * float(R)) ** 2
         assert abs(float(t[5]) - want) < 1e-2, (x, y, R, t[5], want)
+
+
+@pytest.mark.parametrize("ndim", [2, 3])
+@pytest.mark.parametrize("dtype", [np.uint8, np.float32])
+def test_voxels_on_and_at_the_centre_inside_a_band(ndim, dtype):
+    """Radii of half a band and less, whose centre voxel lies inside the bands: on the centre (no
+    direction), off it by less than the Newton steps reach (a direction of length one), and anywhere,
+    against sums in 64 bits."""
+    import torch
+    from paper_1804_06304_gb300 import ac
+    rng = np.random.default_rng(ndim)
+    dims = (20, 17) if ndim == 2 else (12, 11, 10)
+    n, rho = 400, 2.0 ** (-1.0 / ndim)
+    c = np.zeros((n, 3))
+    c[:, :ndim] = rng.random((n, ndim)) * (np.array(dims) - 1)
+    c[:200, :ndim] = np.round(c[:200, :ndim])                         # on a voxel
+    c[:100, 0] = rng.choice([0.0, 1e-15, 3e-15, 1e-14, 1e-20], 100)   # near the first of its row
+    seeds = np.column_stack([c, rng.uniform(0.2, 0.6, n)]).astype(np.float32)
+    image = (rng.random(dims[::-1]) * 200).astype(dtype)
+    C = ac.ac_seed(ac.ac_create_volume(image), explicit=seeds)
+    trace = torch.zeros((1, n, 9), device="cuda")
+    p = ac.EvolveParams(N=1, T=1, eps0=0.0, Rmin=0.1, Rmax=9.0, path=ac.AC_PATH_GRID)
+    ac.ac_evolve(C, p, trace=(trace, 0, n, 1, 2))
+    off = np.stack(np.meshgrid(*[np.arange(-2, 3)] * ndim, indexing="ij"), -1).reshape(-1, ndim)
+    for got, s in zip(trace.cpu().numpy()[0].astype(np.float64), seeds.astype(np.float64)):
+        at, R = s[:ndim], s[3]
+        v = np.round(at).astype(int) + off
+        x = v - at
+        r = np.sqrt((x ** 2).sum(1))
+        keep = r <= R + 0.5
+        v, x, r = v[keep], x[keep], r[keep]
+        I = image[tuple(np.clip(v[:, d], 0, dims[d] - 1) for d in reversed(range(ndim)))].astype(np.float64)
+        t1, t2 = (r - rho * R) / rho + 0.5, r - R + 0.5
+        b1, b2 = (t1 >= 0) & (t1 <= 1), (t2 >= 0) & (t2 <= 1)
+        J = ((-1.0 + 2.0 * np.clip(t1, 0, 1) - np.clip(t2, 0, 1)) * I).sum()
+        slope = np.where(r > 0, (b1 * (-2.0 / rho) + b2) * I / np.maximum(r, 1e-300), 0.0)
+        inv = (2.0 * R) ** -ndim
+        want = np.array([J, ((b1 * -2.0 + b2) * I).sum() - ndim * J / R] + [(slope * x[:, d]).sum() for d in range(ndim)]) * inv
+        np.testing.assert_allclose(got[4:6 + ndim], want, rtol=1e-4, atol=2e-3, err_msg=str(s))
