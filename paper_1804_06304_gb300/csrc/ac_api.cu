@@ -924,15 +924,16 @@ ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets
             const int *sizes = vol->ndim == 3 ? sizes3 : sizes2, n_sizes = vol->ndim == 3 ? 5 : 8;
             const int *sizes_z = vol->ndim == 3 ? sizes3 : one, n_z = vol->ndim == 3 ? 5 : 1;
             const double away = std::min(1.0, p->T / 100.0);
-            auto time_of = [&](double limit) {   // of the current cells' fitted layout, if below the limit
+            // of the current cells' fitted layout, if below the limit: for balls that fit, and with
+            // those that do not
+            auto time_of = [&](double limit, double &with_global) {
                 // a halo cut short sends balls that have grown or moved to global memory (cut by
                 // 1.4 R0: 0.7 % of the contour-iterations of 10, 32 % of 100), and a CTA waits
                 // for its slowest warp
                 const double cut = std::max(0.0, hf - ((h[0] - 2) * (double)vol->sp[0] - 0.5 * p->dR) / r_hint);
                 // balls of the initial radius that leave the region already: within the rest of their
                 // radius of a brick's face, and their warps with them (all of them: 2.7 times the time;
-                // factors of 0.4 to 3 tried on 90 workloads).  Without this, 258x238x76 float at
-                // N = 512 took 2.57 ms, with it 0.98; 60 of the 90 keep their layout.
+                // factors of 0.4 to 3 tried on 90 workloads)
                 double inside = 1.0;
                 for (int d = 0; d < vol->ndim; ++d) {
                     const double out = r_hint + 0.5 * p->dR - (h[d] - 1) * (double)vol->sp[d];
@@ -940,8 +941,10 @@ ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets
                     if (out > 0.0) inside *= 1.0 - std::min(1.0, faces * out / (B[d] * (double)vol->sp[d]));
                 }
                 const double global = inside < 1.0 ? 1.0 - std::pow(inside, per_warp) : 0.0;
-                const double even = estimate(pl.warps, pl.smem) * (1.0 + away * cut * cut) * (1.0 + 1.7 * global);
-                return even * (1.0 - 1e-9) >= limit ? even : even * (0.915 + 0.085 * uneven());
+                const double even = estimate(pl.warps, pl.smem) * (1.0 + away * cut * cut);
+                const double t = even * (1.0 - 1e-9) >= limit ? even : even * (0.915 + 0.085 * uneven());
+                with_global = t * (1.0 + 1.7 * global);
+                return t;
             };
             // the default cells, halved until 1216 bricks come out: kept unless another layout
             // promises 7 % (what the estimate is good for)
@@ -955,8 +958,18 @@ ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets
                 B[dm] = brick_of(dm);
                 nb = count_bricks();
             }
-            int chosen[3] = {cells[0], cells[1], cells[2]};
-            double best = fit(false) ? 0.93 * time_of(1e300) : 1e300;
+            // The best layout for balls that fit is taken unless, with those that do not, another
+            // one promises GAIN against it: few contours hide the global reads well enough
+            // (169x110x139 u16, 3,861 contours: 200 us with most balls outside, 320 us with half).
+            // 258x238x76 float at N = 512 goes from 2.57 to 0.98 ms.
+            constexpr double GAIN = 0.9;
+            int chosen[3] = {cells[0], cells[1], cells[2]}, fitting[3] = {cells[0], cells[1], cells[2]};
+            double best = 1e300, chosen_all = 1e300, best_all = 1e300;
+            if (fit(false)) {
+                best = 0.93 * time_of(1e300, chosen_all);
+                chosen_all *= 0.93;
+                best_all = chosen_all;
+            }
             for (int z = 0; z < n_z; ++z)
                 for (int y = 0; y < n_sizes; ++y)
                     for (int x = 0; x < n_sizes; ++x) {
@@ -965,14 +978,20 @@ ac_status plan_evolve(const ac_volume *vol, const std::vector<SetGeometry> &sets
                         cells[2] = sizes_z[z];
                         if (cells[0] * cells[1] * cells[2] * G > 16 * 32) continue;
                         for (int d = 0; d < vol->ndim; ++d) B[d] = brick_of(d);
-                        if (estimate(warps_of(), 0) >= best || !fit(false)) continue;   // without staging: a lower bound
-                        const double t = time_of(best);
+                        if (estimate(warps_of(), 0) >= best_all || !fit(false)) continue;   // without staging: a lower bound
+                        double all;
+                        const double t = time_of(best_all, all);
                         if (t < best) {
                             best = t;
+                            chosen_all = all;
                             for (int d = 0; d < 3; ++d) chosen[d] = cells[d];
                         }
+                        if (all < best_all) {
+                            best_all = all;
+                            for (int d = 0; d < 3; ++d) fitting[d] = cells[d];
+                        }
                     }
-            for (int d = 0; d < 3; ++d) cells[d] = chosen[d];
+            for (int d = 0; d < 3; ++d) cells[d] = best_all < GAIN * chosen_all ? fitting[d] : chosen[d];
         }
     }
     if (fit(own_bricks)) return AC_OK;
